@@ -33,11 +33,6 @@ METRIC = "converged eigenpairs/s at rel. residual 1e-10, mixed vs FP64 FEAST, 1 
 UNIT = "eigenpairs/s"
 RES_TOL = 1e-10
 FALLBACK_HBM_GBS = 6800.0
-# DRAM bytes (read + write) per group-iteration of each COCG step from one ncu
-# capture (profiles/cocg_steps_laplace3d_64cube.md), valid only for the kernel
-# source they were measured on.
-NCU_TRAFFIC = {"source_sha1": "d111b7a42e3d2659aeb3f935d8e05e73d221142c",
-               "cocg_step_a": (1.108692e9 + 0.626872e9) / 5, "cocg_step_b": (1.181998e9 + 0.467095e9) / 5}
 
 
 def parse():
@@ -107,6 +102,19 @@ def cocg_rates(pr, p):
     gbs_a = bytes_a / (pr["cocg_a_ms"] / 1e3) / 1e9
     gbs_b = bytes_b / (pr["cocg_b_ms"] / 1e3) / 1e9
     return gbs_a, gbs_b
+
+
+def krylov_rate(pr, p):
+    """Algorithmic GB/s of the one-Krylov-space filter of a profiled solve (B = I:
+    one launch per contour pass).  Per step and element of a column tile: the
+    gathered product reads u_j and u_{j-1} and writes s, the orthogonalisation
+    reads s and u_j and writes u_{j+1}, the combination reads u_j once more; the
+    matrix once per step and tile.  Padded columns are not counted."""
+    sc = pr["complex_bytes"] / 2  # the filter's real type
+    live = p.m0 / (pr["groups"] * pr["mt"])
+    mat = p.A.nnz * (4 + sc) + (p.n + 1) * 4
+    nbytes = pr["group_iterations"] * (7 * p.n * pr["mt"] * sc * live + mat)
+    return nbytes / (pr["cocg_a_ms"] / 1e3) / 1e9
 
 
 def fpm_for(pkg, p, mixed, profile):
@@ -348,7 +356,6 @@ def run_gpu(args):
 
     # roofline of the dominant kernel from the per-launch events of the profiled solve
     pr = prof_tot
-    gbs_a, gbs_b = cocg_rates(pr, p)
     peaks_path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     peak, peak_src = FALLBACK_HBM_GBS, "fallback"
     if os.path.exists(peaks_path):
@@ -360,25 +367,21 @@ def run_gpu(args):
                     break
         except (ValueError, OSError):
             pass
-    dom = "cocg_step_a" if pr["cocg_a_ms"] >= pr["cocg_b_ms"] else "cocg_step_b"
-    ach = gbs_b if dom == "cocg_step_b" else gbs_a
-    import hashlib
-
-    src = os.path.join(ROOT, "paper_2002_04807_gb300", "csrc", "k_filter.cu")
-    traffic = None
-    if (hashlib.sha1(open(src, "rb").read()).hexdigest() == NCU_TRAFFIC["source_sha1"] and args.side == 64
-            and dom in NCU_TRAFFIC):
-        launches = pr["cocg_a_launches"] if dom == "cocg_step_a" else pr["cocg_b_launches"]
-        # per launch, averaged like `achieved`: per-group traffic x active groups per launch
-        traffic = NCU_TRAFFIC[dom] * pr["group_iterations"] / max(launches, 1)
-    roofline = {"bound": "hbm", "kernel": dom, "achieved": ach, "peak": peak, "peak_source": peak_src,
-                "unit": "GB/s", "frac": ach / peak, "traffic": traffic,
-                "cocg_step_a_gbs": gbs_a, "cocg_step_b_gbs": gbs_b,
-                "step_a_staged": int(pr.get("step_a_staged", 0)),
-                "step_a_rows_per_item": int(pr.get("step_a_rows_per_item", 0)),
-                "cocg_share_of_step": (pr["cocg_a_ms"] + pr["cocg_b_ms"]) / (ms / args.steps),
-                "timing": "CUDA events around every COCG launch of one extra solve after the timed region "
-                          f"({int(pr['cocg_a_launches'])} step-A launches, {pr['filter_ms']:.0f} ms of filter)"}
+    roofline = {"bound": "hbm", "peak": peak, "peak_source": peak_src, "unit": "GB/s", "traffic": None,
+                "filter_share_of_step": pr["filter_ms"] / (ms / args.steps)}
+    if pr["cocg_b_launches"] == 0:  # one Krylov space per column
+        ach = krylov_rate(pr, p)
+        roofline.update(kernel="krylov_filter", achieved=ach, frac=ach / peak,
+                        timing=f"CUDA events around the {int(pr['cocg_a_launches'])} contour passes of one extra "
+                               f"solve after the timed region ({pr['filter_ms']:.0f} ms of filter)")
+    else:  # COCG per node
+        gbs_a, gbs_b = cocg_rates(pr, p)
+        dom, ach = (("cocg_step_a", gbs_a) if pr["cocg_a_ms"] >= pr["cocg_b_ms"] else ("cocg_step_b", gbs_b))
+        roofline.update(kernel=dom, achieved=ach, frac=ach / peak, cocg_step_a_gbs=gbs_a, cocg_step_b_gbs=gbs_b,
+                        step_a_staged=int(pr.get("step_a_staged", 0)),
+                        step_a_rows_per_item=int(pr.get("step_a_rows_per_item", 0)),
+                        timing="CUDA events around every COCG launch of one extra solve after the timed region "
+                               f"({int(pr['cocg_a_launches'])} step-A launches, {pr['filter_ms']:.0f} ms of filter)")
 
     # end to end through the host C ABI (pinned host buffers, copies inside the timed region)
     e2e = None

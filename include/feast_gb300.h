@@ -35,12 +35,16 @@
  *      fpm(46) inner solver iteration cap (>= 1)
  *      fpm(60) output: total number of inner (COCG) iterations
  *    Library options in reserved slots (0 = automatic):
- *      fpm(50) contour nodes solved at once (node batch); fpm(51) rows per
- *      inner-solver work item (0: the single-problem drivers stage the rows
+ *      fpm(50) contour nodes solved at once (node batch; with B = I and
+ *      fpm(51) = 0 only the unit of fpm(60)'s count: one Krylov space per
+ *      column serves every node, each (node, column) pair stopping at the
+ *      step at which its own COCG solve would); fpm(51) rows per
+ *      inner-solver work item (0: the single-problem drivers take one Krylov
+ *      space per column when B = I, else stage the rows
  *      each item gathers in shared memory, 32 to 64 rows per item, when the
- *      matrix's row blocks read few contiguous column ranges and B is the
- *      identity or diagonal; else 256; > 0: that many rows, gathered through
- *      the caches); fpm(52) seed of the random start block;
+ *      matrix's row blocks read few contiguous column ranges and B is
+ *      diagonal; else 256; > 0: COCG per node on that many rows, gathered
+ *      through the caches); fpm(52) seed of the random start block;
  *      fpm(53) 1 = record per-kernel timings (see feast_last_profile);
  *      fpm(54) arithmetic of the Rayleigh-Ritz projections and Ritz vectors
  *      of the single-problem real and Hermitian drivers: 0 (default) =
@@ -117,17 +121,20 @@ int feast_contour_nodes_rule(int rule, int ne, double emin, double emax, int rat
  * of the calling thread run with fpm(53) = 1 (all zero otherwise; an
  * extreme-eigenvalue search reports the totals of its solves), measured with CUDA events
  * on the solve's stream.  out (host, 20 doubles): [0] ms in COCG step A
- * launches, [1] ms in COCG step B launches, [2] step A launches, [3] step B
- * launches, [4] group-iterations (column groups x COCG steps done), [5] ms in
+ * launches (B = I: in the one-Krylov-space filter, one launch per contour
+ * pass), [1] ms in COCG step B launches (B = I: 0), [2] step A launches, [3]
+ * step B launches, [4] group-iterations (column groups x steps done), [5] ms in
  * filter passes, [6] ms projecting (A Q, Q^T A Q, Q^T B Q), [7] ms in the
  * reduced eigensolver, [8] ms forming Ritz vectors and residuals, [9] tile
  * width W, [10] columns per group mt, [11] n, [12] bytes per complex value,
  * [13] column groups, [14] refinement loops, [15] kernel launches issued,
  * [16] rows per step-A work item, [17] 0 when step A gathers through the
  * caches, 1 when it stages the rows it gathers in shared memory (windows of r
- * copied by the bulk-copy engine), 2 for the staged form with a producer warp
- * and two stages (one CTA per SM), [18] step A CTAs (staged forms), [19]
- * staged rows per row block (staged forms).
+ * copied by the bulk-copy engine; B = I: each CTA keeps its rows of the
+ * vectors there), 2 for the staged form with a producer warp
+ * and two stages (one CTA per SM), [18] step A CTAs (staged forms; B = I: per
+ * column tile), [19] staged rows per row block (staged forms; B = I: rows per
+ * CTA).
  * Library extension (the guide reports phase timings only as a text log).
  * Returns 0. */
 int feast_last_profile(double* out);
@@ -444,7 +451,8 @@ int feast_eig_grad_dev(int n, const int* ia, const int* ja, int m, const double*
  * a CTA that spins there for more than `cycles` SM clock cycles sets an error
  * flag that makes every CTA of the launch return, and the call reports the
  * failure (-3 from the solvers and the reduced-eigensolver entry points) with the
- * context still usable.  The COCG gathering step waits on an mbarrier for the
+ * context still usable.  The one-Krylov-space filter's CTAs meet the same way
+ * after every step; there the solver reports -4.  The COCG gathering step waits on an mbarrier for the
  * bulk copies that stage its rows; a CTA whose wait exceeds the limit sets an
  * error flag, lets its copies in flight land (waiting up to about a second
  * more) and returns, and the solver reports -4 (message in feast_last_error).

@@ -332,6 +332,9 @@ struct Plan {
     int nslot = 1;  // partial-sum slots per group (item slots + bucket slots)
     int nbk = 1;    // bucket counters per group
     size_t gpart = 0, rpart = 0;
+    // one Krylov space per column for all nodes (lzc.teams > 0: B = I and the basis
+    // fits): the cached form for any matrix, the resident form for short rows
+    KrylovPlan lzc, lzr;
 };
 
 struct Bufs {
@@ -371,9 +374,16 @@ struct Bufs {
     int* ozex = nullptr;  // column exponents of the sliced projections
     void* ozw = nullptr;  // exponents and slices of the sliced Ritz-vector product
     void* eig = nullptr;
+    // one Krylov space per column (P.lzc.teams > 0)
+    KrylovArgs lz = {};
+    const KrylovPlan* lzp = nullptr;  // the form chosen for the matrix
+    char* lzmem = nullptr;
 };
 
 size_t cplx_bytes(const Plan& P) { return P.fp64 ? 16 : 8; }
+
+// Device memory a contour pass may take for its Krylov bases.
+constexpr double kKrylovBytes = 64e9;
 
 Plan make_plan(int n, int nnzA, int nnzB, int m0, const int* fpm, bool filter_only = false)
 {
@@ -405,6 +415,13 @@ Plan make_plan(int n, int nnzA, int nnzB, int m0, const int* fpm, bool filter_on
     const int wslots = P.win ? num_sms() * 4 : 0;
     P.nslot = std::max({part_slots(P.nrb), part_slots(P.nrb_b), part_slots(wslots)});
     P.nbk = std::max({part_buckets(P.nrb), part_buckets(P.nrb_b), part_buckets(wslots)});
+    // B = I: one Krylov space per column serves every node (k_krylov.cu); COCG
+    // per node otherwise, when the basis of fpm(46) steps does not fit, and for
+    // callers that set the rows per work item of the COCG steps
+    if (!P.hasB && fpm[50] == 0) {
+        P.lzc = krylov_plan(P.fp64, false, n, m0, P.ne, fpm[45], kKrylovBytes);
+        P.lzr = krylov_plan(P.fp64, true, n, m0, P.ne, fpm[45], kKrylovBytes);
+    }
     if (!filter_only) {
         P.oz = fpm[53] == 0;
         P.gpart = P.oz ? gram_oz_partial_doubles(n, m0, nullptr, nullptr, num_sms())
@@ -431,12 +448,13 @@ struct Carver {
 size_t carve(const Plan& P, void* base, Bufs& B, bool filter_only = false)
 {
     Carver c(base);
-    const size_t vec = (size_t)P.G * P.n * P.W * cplx_bytes(P);
+    const bool lz = P.lzc.teams > 0;
+    const size_t vec = lz ? 0 : (size_t)P.G * P.n * P.W * cplx_bytes(P);
     B.r = c.take<char>(vec);
     B.p0 = c.take<char>(vec);
     B.p1 = c.take<char>(vec);
     B.cs = c.take<ColState>((size_t)P.G * P.W);
-    B.part = c.take<double>((size_t)P.G * P.nslot * P.W * 4);
+    B.part = c.take<double>(lz ? 0 : (size_t)P.G * P.nslot * P.W * 4);
     B.grp_count = c.take<unsigned>(P.G);
     B.bk_count = c.take<unsigned>((size_t)P.G * P.nbk);
     B.grp_done = c.take<int>(P.G);
@@ -446,13 +464,19 @@ size_t carve(const Plan& P, void* base, Bufs& B, bool filter_only = false)
     B.probs = c.take<FiltProb>(1);
     const size_t pk = P.fp64 ? 16 : 8;
     B.app = c.take<int>((size_t)P.n + 1);
-    B.apk = c.take<char>(((size_t)P.nnzA + 7 * (size_t)P.n) * pk);
+    B.apk = c.take<char>(((size_t)P.nnzA + (lz ? 8 : 7) * (size_t)P.n) * pk);
     if (P.hasB) {
         B.bpp = c.take<int>((size_t)P.n + 1);
         B.bpk = c.take<char>(((size_t)P.nnzB + 7 * (size_t)P.n) * pk);
         B.bd = c.take<double>((size_t)P.n);
     }
-    if (P.win) {
+    if (lz) {
+        KrylovArgs t = {};
+        const size_t bc = krylov_layout(P.lzc, nullptr, t);
+        const size_t br = P.lzr.teams > 0 ? krylov_layout(P.lzr, nullptr, t) : 0;
+        B.lzmem = c.take<char>(std::max(bc, br));
+    }
+    if (P.win && !lz) {
         const size_t nrb32 = ((size_t)P.n + 31) / 32;
         // per row block its local row pointers ((rows + 4) ints: at most 36 per 32 rows
         // for 32- to 80-row blocks, plus one block) and its packed entries
@@ -461,7 +485,7 @@ size_t carve(const Plan& P, void* base, Bufs& B, bool filter_only = false)
         B.wwin = c.take<int2>(nrb32 * kWinMax);
         B.wstat = c.take<int>(4);
     }
-    B.dQ = c.take<char>((size_t)P.G * P.mt * P.n * (P.fp64 ? 8 : 4));
+    B.dQ = c.take<char>(lz ? 0 : (size_t)P.G * P.mt * P.n * (P.fp64 ? 8 : 4));
     B.zw = c.take<double>(4 * (size_t)P.ne);
     if (filter_only) return c.off + 256;
     const size_t blk = (size_t)P.n * P.m0;
@@ -663,11 +687,46 @@ struct Csr {
     const double* v = nullptr;
 };
 
+// One filter pass from one Krylov space per column (B = I), a single launch.
+int krylov_pass(const Plan& P, Bufs& B, int rii, const double* R, const double* X, double tol, cudaStream_t s)
+{
+    KrylovArgs a = B.lz;
+    a.probs = B.probs;
+    a.units = nullptr;
+    a.nunits = (P.m0 + B.lzp->cols - 1) / B.lzp->cols;
+    a.nbp = P.nbp;
+    a.nbatch = P.nbatch;
+    a.rii = rii;
+    a.tol2 = tol * tol;
+    a.err = B.groups_left + 1;
+    a.limit = wait_limit_cycles();
+    a.R = R;
+    a.X = X;
+    a.Q = B.Q;
+    a.iter_max = B.iter_max;
+    a.work = B.work;
+    CK(cudaMemsetAsync(B.iter_max, 0, sizeof(int) * P.nbatch, s));
+    CK(cudaMemsetAsync(a.err, 0, sizeof(int), s));
+    CK(cudaMemsetAsync(a.bar, 0, sizeof(unsigned) * ((size_t)a.nteams * 32 + 32), s));
+    const size_t e0 = g_prof.on ? g_prof.mark(s) : 0;
+    CK(launch_krylov_filter(a, *B.lzp, P.fp64, s));
+    if (g_prof.on) g_prof.a.push_back({e0, g_prof.mark(s)});
+    int werr = 0;
+    CK(cudaMemcpyAsync(&werr, a.err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    if (werr) {
+        g_err = "contour filter: a wait of the Krylov steps exceeded the wait limit";
+        return -4;
+    }
+    return 0;
+}
+
 // One filter pass (all node batches) into B.Q.  rii selects the right-hand
 // side R (device row-major n x m0 in B.Y) and the coefficients.
 int filter_pass(const Plan& P, Bufs& B, int rii, const double* R, const double* X, int maxit, double tol,
                 cudaStream_t s)
 {
+    if (P.lzc.teams > 0) return krylov_pass(P, B, rii, R, X, tol, s);
     FilterArgs fa;
     memset(&fa, 0, sizeof(fa));
     fa.probs = B.probs;
@@ -873,20 +932,54 @@ int choose_step_a(const Plan& P, Bufs& B, cudaStream_t s)
     return 0;
 }
 
+// Form and matrix of the Krylov steps: rows of at most eight entries are packed
+// in the order the steps load them, and the CTAs keep their rows of the vectors
+// in shared memory when they fit; other matrices are packed in the chunks of
+// pack_matrix and gathered through the caches.
+int setup_krylov(const Plan& P, Bufs& B, const Csr& A, cudaStream_t s)
+{
+    B.bmode = 0;
+    B.wrb = 0;
+    B.wws = false;
+    int wide = 1;
+    if ((long long)A.nnz <= 8LL * A.n) {
+        int* d_wide = (int*)B.lzmem;
+        CK(cudaMemsetAsync(d_wide, 0, sizeof(int), s));
+        CK(launch_krylov_scan(A.n, A.ia, A.ja, d_wide, s));
+        CK(cudaMemcpyAsync(&wide, d_wide, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+    }
+    B.lzp = wide || P.lzr.teams == 0 || P.lzc.cost < P.lzr.cost ? &P.lzc : &P.lzr;
+    krylov_layout(*B.lzp, B.lzmem, B.lz);
+    B.lz.one_chunk = wide ? 0 : 1;
+    B.RB = B.lzp->resident ? 64 : 256;
+    if (!wide) {
+        CK(launch_krylov_pack(A.n, B.lzp->rpc, A.ia, A.ja, A.v, P.fp64, B.apk, s));
+        return 0;
+    }
+    int amode = 0;
+    return pack_matrix(A, P.fp64, false, B.app, B.apk, nullptr, &amode, s);
+}
+
 int setup_filter(const Plan& P, Bufs& B, const Csr& A, const Csr& Bm, const std::vector<double>& zw,
                  const double* lam, const int* mk, cudaStream_t s)
 {
     CK(cudaMemcpyAsync(B.zw, zw.data(), sizeof(double) * zw.size(), cudaMemcpyHostToDevice, s));
-    int amode = 0;
-    int st = pack_matrix(A, P.fp64, false, B.app, B.apk, nullptr, &amode, s);
-    if (st) return st;
-    B.bmode = 0;
-    if (P.hasB) {
-        st = pack_matrix(Bm, P.fp64, true, B.bpp, B.bpk, B.bd, &B.bmode, s);
+    int amode = 0, st = 0;
+    if (P.lzc.teams > 0) {
+        st = setup_krylov(P, B, A, s);
+        if (st) return st;
+    } else {
+        st = pack_matrix(A, P.fp64, false, B.app, B.apk, nullptr, &amode, s);
+        if (st) return st;
+        B.bmode = 0;
+        if (P.hasB) {
+            st = pack_matrix(Bm, P.fp64, true, B.bpp, B.bpk, B.bd, &B.bmode, s);
+            if (st) return st;
+        }
+        st = choose_step_a(P, B, s);
         if (st) return st;
     }
-    st = choose_step_a(P, B, s);
-    if (st) return st;
     FiltProb fp;
     memset(&fp, 0, sizeof(fp));
     fp.n = P.n;
@@ -1135,16 +1228,18 @@ int run_feast(const Plan& P, Bufs& B, const Csr& A, const Csr& Bm, int* fpm, dou
         o[3] = (double)g_prof.b.size();
         o[4] = (double)work;
         for (auto& ph : g_prof.phase) o[5 + ph.first] += g_prof.ms(ph.second.first, ph.second.second);
-        o[9] = (double)P.W;
-        o[10] = (double)P.mt;
+        const KrylovPlan* lzp = B.lzp;
+        o[9] = (double)(lzp ? lzp->cols : P.W);
+        o[10] = (double)(lzp ? lzp->cols : P.mt);
         o[11] = (double)P.n;
         o[12] = (double)cplx_bytes(P);
-        o[13] = (double)P.G;
+        o[13] = (double)(lzp ? (P.m0 + lzp->cols - 1) / lzp->cols : P.G);
         o[14] = (double)k;
         o[16] = (double)B.RB;
-        o[17] = B.wws ? 2.0 : (B.wrb ? 1.0 : 0.0);
-        o[18] = (double)(B.wrb ? B.wgrid : 0);
-        o[19] = (double)(B.wrb ? B.wcapr : 0);
+        const bool res = lzp && lzp->resident;
+        o[17] = B.wws ? 2.0 : (B.wrb || res ? 1.0 : 0.0);
+        o[18] = (double)(B.wrb ? B.wgrid : (res ? lzp->nc : 0));
+        o[19] = (double)(B.wrb ? B.wcapr : (res ? lzp->rpc : 0));
     }
     return info;
 }

@@ -158,6 +158,53 @@ cudaError_t launch_cocg_step_aw(const FilterArgs& a, bool fp64, int rbw, int k, 
 size_t ws_smem_bytes(int W, int rbw, int capr, int cape);
 int ws_occupancy(bool fp64, int W, int bmode, int rbw, int groups, size_t smem);
 cudaError_t launch_cocg_step_ws(const FilterArgs& a, int rbw, int k, int grid, size_t smem, cudaStream_t s);
+// ---------------------------------------------------------------- one Krylov space for all nodes (k_krylov.cu)
+struct KrylovPlan {
+    int teams = 0;  // teams of CTAs at once; 0: the basis does not fit the given memory
+    int nc = 0;     // CTAs per team
+    bool resident = false;  // the CTAs keep their rows of two vectors in shared memory
+    int rpc = 0;    // rows per CTA (resident form)
+    int lanes = 0;  // 16-byte lanes per tile row
+    int cols = 0;   // columns per tile
+    int nl = 0;     // nodes solved at once per column
+    int ne = 0, maxit = 0;
+    size_t slot_vecs = 0, team_bytes = 0;
+    double cost = 0.0;  // estimated time of one step for all columns
+};
+struct KrylovArgs {
+    const FiltProb* probs;
+    const int2* units;  // (problem, tile) of every work unit, nullptr: tile u of problem 0
+    int nunits, nteams, nc;
+    int ne, nl, maxit, nbp, nbatch;
+    int rii;
+    int one_chunk;      // rows of at most eight entries, packed by krylov_pack (entries of row i at 8 i)
+    double tol2;
+    size_t slot_vecs, team_bytes;
+    char* basis;        // [team][maxit + 1][slot_vecs] 16-byte vectors
+    void* part;         // [team][2][nc][cols] partial sums (8 bytes)
+    double* coef;       // [team][2][maxit + 2][cols] alpha_j, beta_{j+1}
+    void* g;            // [team][maxit][cols] combination coefficients (filter precision)
+    float4* pair;       // [team][ne][cols]
+    int* kstop;         // [team][ne][cols]
+    double2* piv;       // [team][cols][maxit][nl]
+    unsigned* bar;      // [team][32], zeroed
+    int* mail;          // [team][32]
+    unsigned* queue;    // zeroed
+    int* err;           // zeroed; 1 when a CTA gave up waiting
+    long long limit;
+    const double* R;
+    const double* X;
+    double* Q;
+    int* iter_max;      // [problem][nbatch]
+    unsigned long long* work;
+};
+KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes);
+size_t krylov_layout(const KrylovPlan& k, char* base, KrylovArgs& a);
+cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, cudaStream_t s);
+cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, bool fp64, void* out,
+                               cudaStream_t s);
+cudaError_t launch_krylov_filter(const KrylovArgs& a, const KrylovPlan& p, bool fp64, cudaStream_t s);
+
 // persistent grid size of the COCG kernels: SMs x resident CTAs per SM
 int filter_grid(bool fp64, int W);
 void filter_grids(bool fp64, int W, int* grid_a, int* grid_b);
