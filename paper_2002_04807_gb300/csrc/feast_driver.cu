@@ -382,8 +382,10 @@ struct Bufs {
 
 size_t cplx_bytes(const Plan& P) { return P.fp64 ? 16 : 8; }
 
-// Device memory a contour pass may take for its Krylov bases.
+// Device memory a contour pass may take for its Krylov bases, of one problem and
+// of a batch (which allocates per call).
 constexpr double kKrylovBytes = 64e9;
+constexpr double kKrylovBatchBytes = 8e9;
 
 Plan make_plan(int n, int nnzA, int nnzB, int m0, const int* fpm, bool filter_only = false)
 {
@@ -2296,12 +2298,58 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         nnzA += (long long)aja[p].size();
         nnzB += (long long)bja[p].size();
         ppA += n + 1;
-        pkA += (long long)aja[p].size() + 7LL * n;
+        pkA += std::max((long long)aja[p].size() + 7LL * n, 8LL * n);
         if (bmode == 2) {
             ppB += n + 1;
             pkB += (long long)bja[p].size() + 7LL * n;
         }
         maxm = std::max(maxm, m);
+    }
+    // B = I: one Krylov space per column (k_krylov.cu), when every row packs into
+    // eight entries; problems of similar size share a launch (kinds), the
+    // largest first
+    struct Kind {
+        KrylovPlan plan;
+        KrylovArgs args = {};
+        std::vector<int> probs;
+    };
+    std::vector<Kind> kinds;
+    size_t lz_bytes = 0;
+    if (!hasB && fpm[50] == 0) {
+        bool fits = true;
+        for (int p = 0; p < np && fits; ++p)
+            for (int i = 0; i < probs[p].n && fits; ++i) {
+                const int len = aia[p][i + 1] - aia[p][i];
+                const int* c = aja[p].data() + aia[p][i];
+                fits = len < 8 || (len == 8 && std::find(c, c + len, i) != c + len);
+            }
+        std::vector<int> order(np);
+        for (int p = 0; p < np; ++p) order[p] = p;
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return probs[x].n > probs[y].n; });
+        for (int q = 0; q < np && fits;) {
+            // from the largest problem left, those of more than half its rows (all
+            // the rest once one CTA holds a four-column tile)
+            const int top = probs[order[q]].n, least = top > 6912 ? top / 2 : 0;
+            Kind kd;
+            std::vector<int> kn, km;
+            for (; q < np && probs[order[q]].n > least; ++q) {
+                kd.probs.push_back(order[q]);
+                kn.push_back(probs[order[q]].n);
+                km.push_back(probs[order[q]].m0);
+            }
+            kd.plan = krylov_plan_set(fp64, (int)kn.size(), kn.data(), km.data(), ne, maxit, kKrylovBatchBytes);
+            fits = kd.plan.teams > 0;
+            if (fits) lz_bytes = std::max(lz_bytes, krylov_layout(kd.plan, nullptr, kd.args));
+            kinds.push_back(std::move(kd));
+        }
+        if (!fits) kinds.clear();
+    }
+    const bool lz = !kinds.empty();
+    long long max_units = 0;
+    for (const Kind& kd : kinds) {
+        long long u = 0;
+        for (const int p : kd.probs) u += (probs[p].m0 + kd.plan.cols - 1) / kd.plan.cols;
+        max_units = std::max(max_units, u);
     }
     int ga = 1, gb = 1;
     filter_grids(fp64, W, &ga, &gb);
@@ -2339,9 +2387,9 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         (void)bump.take<double>(bmode == 1 ? rows : 0);
         (void)bump.take<FiltProb>(np);
         (void)bump.take<BProb>(np);
-        (void)bump.take<char>(vec * csz * 3);
-        (void)bump.take<ColState>(colo);
-        (void)bump.take<double>((size_t)grpo * nslot * W * 4);
+        (void)bump.take<char>(lz ? 0 : vec * csz * 3);
+        (void)bump.take<ColState>(lz ? 0 : colo);
+        (void)bump.take<double>(lz ? 0 : (size_t)grpo * nslot * W * 4);
         (void)bump.take<unsigned>((size_t)grpo * nbk);
         (void)bump.take<unsigned>(grpo);
         (void)bump.take<int>(grpo);
@@ -2350,7 +2398,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         (void)bump.take<unsigned long long>(1);
         (void)bump.take<int>(1);
         (void)bump.take<double>((size_t)np * ne * 4);
-        (void)bump.take<char>(dqo * (fp64 ? 8 : 4));
+        (void)bump.take<char>(lz ? 0 : dqo * (fp64 ? 8 : 4));
         for (int t = 0; t < 6; ++t) (void)bump.take<double>(qo);  // Y, Q, X, T, T2, xc
         for (int t = 0; t < 3; ++t) (void)bump.take<double>(co);  // Aq, Bq, Vr
         (void)bump.take<double>(lo);
@@ -2363,6 +2411,8 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         (void)bump.take<double>(wo);
         (void)bump.take<int>(items_a_max);
         (void)bump.take<int>(items_b);
+        (void)bump.take<char>(lz_bytes);
+        (void)bump.take<int2>(max_units);
         if (pass == 0) {
             cudaError_t e = dm.alloc(&base, bump.off + 4096);
             if (e != cudaSuccess) return cuda_fail(e, "batched workspace");
@@ -2383,9 +2433,9 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
     double* d_bd = bump.take<double>(bmode == 1 ? rows : 0);
     FiltProb* d_fp = bump.take<FiltProb>(np);
     BProb* d_bp = bump.take<BProb>(np);
-    char* d_vec = bump.take<char>(vec * csz * 3);
-    ColState* d_cs = bump.take<ColState>(colo);
-    double* d_part = bump.take<double>((size_t)grpo * nslot * W * 4);
+    char* d_vec = bump.take<char>(lz ? 0 : vec * csz * 3);
+    ColState* d_cs = bump.take<ColState>(lz ? 0 : colo);
+    double* d_part = bump.take<double>(lz ? 0 : (size_t)grpo * nslot * W * 4);
     unsigned* d_bkcount = bump.take<unsigned>((size_t)grpo * nbk);
     unsigned* d_gcount = bump.take<unsigned>(grpo);
     int* d_gdone = bump.take<int>(grpo);
@@ -2394,7 +2444,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
     unsigned long long* d_work = bump.take<unsigned long long>(1);
     int* d_k = bump.take<int>(1);
     double* d_zw = bump.take<double>((size_t)np * ne * 4);
-    char* d_dq = bump.take<char>(dqo * (fp64 ? 8 : 4));
+    char* d_dq = bump.take<char>(lz ? 0 : dqo * (fp64 ? 8 : 4));
     double* d_Y = bump.take<double>(qo);
     double* d_Q = bump.take<double>(qo);
     double* d_X = bump.take<double>(qo);
@@ -2414,6 +2464,13 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
     double* d_rwork = bump.take<double>(wo);
     int* d_itp = bump.take<int>(items_a_max);
     int* d_itpb = bump.take<int>(items_b);
+    char* d_lz = bump.take<char>(lz_bytes);
+    int2* d_units = bump.take<int2>(max_units);
+    std::vector<int> rpc(np, 0);  // rows per CTA of each problem's resident form
+    for (Kind& kd : kinds) {
+        krylov_layout(kd.plan, d_lz, kd.args);
+        for (const int p : kd.probs) rpc[p] = krylov_rows(probs[p].n, kd.plan.nc);
+    }
     cudaStream_t s = nullptr;
     CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     struct StreamGuard {
@@ -2435,12 +2492,16 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
             f.ia = b.ia = d_ia + oa;
             f.ja = b.ja = d_ja + onz;
             f.av = b.av = d_a + onz;
-            // padded chunk pointers from the host copy
-            std::vector<int> pp(n + 1, 0);
-            for (int i = 0; i < n; ++i) pp[i + 1] = pp[i] + (aia[p][i + 1] - aia[p][i] + 7) / 8 * 8;
-            CK(cudaMemcpyAsync(d_app + opp, pp.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s));
-            CK(cudaStreamSynchronize(s));
-            CK(launch_pack_csr(n, d_ia + oa, d_ja + onz, d_a + onz, d_app + opp, fp64, d_apk + opk * pkz, s));
+            if (lz) {
+                CK(launch_krylov_pack(n, rpc[p], d_ia + oa, d_ja + onz, d_a + onz, fp64, d_apk + opk * pkz, s));
+            } else {
+                // padded chunk pointers from the host copy
+                std::vector<int> pp(n + 1, 0);
+                for (int i = 0; i < n; ++i) pp[i + 1] = pp[i] + (aia[p][i + 1] - aia[p][i] + 7) / 8 * 8;
+                CK(cudaMemcpyAsync(d_app + opp, pp.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s));
+                CK(cudaStreamSynchronize(s));
+                CK(launch_pack_csr(n, d_ia + oa, d_ja + onz, d_a + onz, d_app + opp, fp64, d_apk + opk * pkz, s));
+            }
             f.app = d_app + opp;
             f.apk = d_apk + opk * pkz;
             if (hasB) {
@@ -2470,7 +2531,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
             oa += n + 1;
             onz += (long long)aja[p].size();
             opp += n + 1;
-            opk += (long long)aja[p].size() + 7LL * n;
+            opk += std::max((long long)aja[p].size() + 7LL * n, 8LL * n);
             std::vector<double> zw;
             contour(fpm[15], ne, probs[p].emin, probs[p].emax, fpm[17] / 100.0, zw);
             std::copy(zw.begin(), zw.end(), zw_all.begin() + (size_t)p * ne * 4);
@@ -2613,7 +2674,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
     };
     // ---- autotuner: time step A (first step, no state change) for a few
     // rows-per-item choices on this batch, keep the fastest
-    if (fpm[50] == 0) {
+    if (fpm[50] == 0 && !lz) {
         const long long key = (rows >> 16) * 64 + W * 2 + (fp64 ? 1 : 0);
         int cached = 0;
         {
@@ -2657,8 +2718,53 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         // the timing runs reset Q: start again from the start blocks
         CK(cudaMemcpyAsync(d_Q, d_Y, sizeof(double) * qo, cudaMemcpyDeviceToDevice, s));
     }
-    st = capture_chunk();
-    if (st) return st;
+    if (!lz) {
+        st = capture_chunk();
+        if (st) return st;
+    }
+    // ---- one contour pass over the unfinished problems, a launch per kind
+    std::vector<int2> units;
+    std::vector<int> itmax((size_t)np * nbatch);
+    auto krylov_pass = [&]() -> int {
+        CK(cudaMemsetAsync(d_itmax, 0, sizeof(int) * (size_t)np * nbatch, s));
+        for (Kind& kd : kinds) {
+            units.clear();
+            for (const int p : kd.probs)
+                if (!done[p])
+                    for (int t = 0; t * kd.plan.cols < probs[p].m0; ++t) units.push_back(make_int2(p, t));
+            if (units.empty()) continue;
+            KrylovArgs a = kd.args;
+            a.probs = d_fp;
+            a.units = d_units;
+            a.nunits = (int)units.size();
+            a.nbp = nbp;
+            a.nbatch = nbatch;
+            a.rii = 1;
+            a.one_chunk = 1;
+            a.tol2 = tol * tol;
+            a.err = d_k;
+            a.limit = wait_limit_cycles();
+            a.R = d_Y;
+            a.X = d_X;
+            a.Q = d_Q;
+            a.iter_max = d_itmax;
+            a.work = d_work;
+            CK(cudaMemcpyAsync(d_units, units.data(), sizeof(int2) * units.size(), cudaMemcpyHostToDevice, s));
+            CK(cudaMemsetAsync(a.err, 0, sizeof(int), s));
+            CK(cudaMemsetAsync(a.bar, 0, sizeof(unsigned) * ((size_t)a.nteams * 32 + 32), s));
+            CK(launch_krylov_filter(a, kd.plan, fp64, s));
+            int werr = 0;
+            CK(cudaMemcpyAsync(&werr, a.err, sizeof(int), cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));  // and the unit list may be rebuilt
+            if (werr) {
+                g_err = "contour filter: a wait of the Krylov steps exceeded the wait limit";
+                return -4;
+            }
+        }
+        CK(cudaMemcpyAsync(itmax.data(), d_itmax, sizeof(int) * itmax.size(), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        return 0;
+    };
     // ---- Rayleigh-Ritz graph
     {
         cudaGraph_t graph;
@@ -2729,6 +2835,15 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         CK(cudaMemcpyAsync(d_fp, fpv.data(), sizeof(FiltProb) * np, cudaMemcpyHostToDevice, s));
         if (!left) break;
         // residual-inverse filter pass over the unfinished problems
+        if (lz) {
+            { const int kp = krylov_pass(); if (kp) return kp; }
+            for (int b = 0; b < nbatch; ++b) {
+                int most = 0;
+                for (int p = 0; p < np; ++p) most = std::max(most, itmax[(size_t)p * nbatch + b]);
+                total_steps += most;
+            }
+            continue;
+        }
         { const int sg = set_groups(); if (sg) return sg; }
         int g_a, g_b, g_i;
         grids(g_a, g_b, g_i);

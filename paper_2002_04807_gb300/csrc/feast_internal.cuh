@@ -199,6 +199,8 @@ struct KrylovArgs {
     unsigned long long* work;
 };
 KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes);
+KrylovPlan krylov_plan_set(bool fp64, int np, const int* n, const int* m, int ne, int maxit, double max_bytes);
+int krylov_rows(int n, int nc);  // rows per CTA of the resident form
 size_t krylov_layout(const KrylovPlan& k, char* base, KrylovArgs& a);
 cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, cudaStream_t s);
 cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, bool fp64, void* out,

@@ -890,19 +890,33 @@ cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, con
 }
 
 // ---------------------------------------------------------------- plan and launch
+int krylov_rows(int n, int nc) { return krylov_rpc(n, nc); }
+
 // Bytes of Krylov bases beyond which a pass takes its tiles one team at a time.
 static constexpr double kKrylovMany = 16e9;
 
-// Microseconds of one step for all columns, by the measured parts of a step on
+// Microseconds of one step of a tile of an n-row problem, by the measured parts of a step on
 // GB300: a pass of 512 lanes through both phases (resident 1.2, cached 2.9 with
 // two CTAs per SM, each times 4 in FP64), and the two sums of a step (2.2 within
 // a CTA; 6 across a team and more with its size).
-static double krylov_cost(const KrylovPlan& k, bool fp64, int n, int m)
+static double krylov_tile_cost(const KrylovPlan& k, bool fp64, int n)
 {
-    const int units = (m + k.cols - 1) / k.cols, rounds = (units + k.teams - 1) / k.teams;
-    const int rows = k.resident ? k.rpc : ((n + kLzBlock - 1) / kLzBlock + k.nc - 1) / k.nc * kLzBlock;
+    const int rows = k.resident ? krylov_rpc(n, k.nc) : ((n + kLzBlock - 1) / kLzBlock + k.nc - 1) / k.nc * kLzBlock;
     const double passes = std::ceil((double)rows * k.lanes / kLzThreads);
-    return rounds * (1.8 + passes * (k.resident ? 1.2 : 2.9) * (fp64 ? 4.0 : 1.0) + (k.nc == 1 ? 2.2 : 6.0 + 0.035 * k.nc));
+    return 1.8 + passes * (k.resident ? 1.2 : 2.9) * (fp64 ? 4.0 : 1.0) + (k.nc == 1 ? 2.2 : 6.0 + 0.035 * k.nc);
+}
+
+// The parts of a plan that follow from its width, for problems of at most n rows.
+static double krylov_size(KrylovPlan& k, bool fp64, int lanes, int n, int ne, int maxit)
+{
+    k.lanes = lanes;
+    k.cols = lanes * (fp64 ? 2 : 4);
+    k.nl = std::min(ne, 32);
+    k.maxit = maxit;
+    k.ne = ne;
+    k.slot_vecs = (size_t)n * lanes;
+    k.team_bytes = ((size_t)maxit + 1) * k.slot_vecs * 16;
+    return (double)k.team_bytes + (double)k.cols * k.nl * 16.0 * maxit + (double)k.cols * (24.0 * maxit + 20.0 * ne);
 }
 
 KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes)
@@ -913,14 +927,7 @@ KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit
         if (!resident && lanes != kLzMaxLanes) break;
         KrylovPlan k;
         k.resident = resident;
-        k.lanes = lanes;
-        k.cols = lanes * (fp64 ? 2 : 4);
-        k.nl = std::min(ne, 32);
-        k.maxit = maxit;
-        k.ne = ne;
-        k.slot_vecs = (size_t)n * lanes;
-        k.team_bytes = ((size_t)maxit + 1) * k.slot_vecs * 16;
-        const double per_team = (double)k.team_bytes + (double)k.cols * k.nl * 16.0 * maxit + (double)k.cols * (24.0 * maxit + 20.0 * ne);
+        const double per_team = krylov_size(k, fp64, lanes, n, ne, maxit);
         if (per_team > max_bytes) continue;
         const int units = (m + k.cols - 1) / k.cols;
         const int fit = (int)std::max(1.0, kKrylovMany / per_team);
@@ -930,9 +937,40 @@ KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit
                 k.nc = one ? 1 : std::max(1, std::min(ctas / t, (n + 63) / 64));
                 k.rpc = resident ? krylov_rpc(n, k.nc) : 0;
                 if ((size_t)k.rpc * lanes * 32 > kLzSmem) continue;
-                k.cost = krylov_cost(k, fp64, n, m);
+                k.cost = ((units + t - 1) / t) * krylov_tile_cost(k, fp64, n);
                 if (best.teams == 0 || k.cost < best.cost) best = k;
             }
+    }
+    return best;
+}
+
+// Plan of the resident form for a set of problems (np of them, n[i] rows and
+// m[i] columns) whose tiles the teams take from one queue; teams = 0 when the
+// largest does not fit.
+KrylovPlan krylov_plan_set(bool fp64, int np, const int* n, const int* m, int ne, int maxit, double max_bytes)
+{
+    KrylovPlan best;
+    const int sms = num_sms(), maxn = *std::max_element(n, n + np);
+    for (int lanes = kLzMaxLanes; lanes >= 1; lanes /= 2) {
+        KrylovPlan k;
+        k.resident = true;
+        const double per_team = krylov_size(k, fp64, lanes, maxn, ne, maxit);
+        if (per_team > max_bytes) continue;
+        long long units = 0;
+        for (int i = 0; i < np; ++i) units += (m[i] + k.cols - 1) / k.cols;
+        for (k.nc = 1; k.nc <= sms; k.nc *= 2) {
+            k.rpc = krylov_rpc(maxn, k.nc);
+            if ((size_t)k.rpc * lanes * 32 > kLzSmem) continue;
+            k.teams = (int)std::min<double>({(double)(sms / k.nc), (double)units, std::max(1.0, max_bytes / per_team)});
+            double sum = 0.0, longest = 0.0;
+            for (int i = 0; i < np; ++i) {
+                const double us = krylov_tile_cost(k, fp64, n[i]);
+                sum += us * ((m[i] + k.cols - 1) / k.cols);
+                longest = std::max(longest, us);
+            }
+            k.cost = std::max(longest, sum / k.teams + 0.5 * longest);
+            if (best.teams == 0 || k.cost < best.cost) best = k;
+        }
     }
     return best;
 }
