@@ -2246,6 +2246,13 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
     std::vector<FiltProb> fpv(np);
     std::vector<BProb> bpv(np);
     std::vector<int> G(np);
+    // rows per split of the Gram products: eight blocks per SM over the whole batch
+    double tile_rows = 0.0;
+    for (int p = 0; p < np; ++p) {
+        const int T = (probs[p].m0 + 63) / 64;
+        tile_rows += (double)probs[p].n * (T * (T + 1) / 2);
+    }
+    const int gram_rows = (int)std::min(4096.0, std::max(256.0, tile_rows / (8.0 * num_sms())));
     long long rows = 0, vec = 0, qo = 0, dqo = 0, co = 0, gpo = 0, wo = 0, nnzA = 0, nnzB = 0, ppA = 0, pkA = 0,
               ppB = 0, pkB = 0;
     int colo = 0, grpo = 0, lo = 0, gram_b = 0, gemm_b = 0, res_b = 0, maxm = 0;
@@ -2274,7 +2281,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         b.c_off = co;
         b.l_off = lo;
         b.gram_T = (m + 63) / 64;
-        b.gram_ks = std::max(1, std::min(32, (n + 4095) / 4096));
+        b.gram_ks = std::max(1, std::min(64, (n + gram_rows - 1) / gram_rows));
         b.gram_b0 = gram_b;
         b.gpart_off = gpo;
         b.gemm_b0 = gemm_b;
@@ -2413,6 +2420,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         (void)bump.take<int>(items_b);
         (void)bump.take<char>(lz_bytes);
         (void)bump.take<int2>(max_units);
+        (void)bump.take<char>(jacobi_batch_bytes(np));
         if (pass == 0) {
             cudaError_t e = dm.alloc(&base, bump.off + 4096);
             if (e != cudaSuccess) return cuda_fail(e, "batched workspace");
@@ -2466,6 +2474,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
     int* d_itpb = bump.take<int>(items_b);
     char* d_lz = bump.take<char>(lz_bytes);
     int2* d_units = bump.take<int2>(max_units);
+    char* d_jwork = bump.take<char>(jacobi_batch_bytes(np));
     std::vector<int> rpc(np, 0);  // rows per CTA of each problem's resident form
     for (Kind& kd : kinds) {
         krylov_layout(kd.plan, d_lz, kd.args);
@@ -2642,16 +2651,14 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         return 0;
     };
     // ---- COCG chunk graph: (step A, step B, k += 1) x 8, step index on the device
-    cudaGraphExec_t chunk_exec = nullptr, rr_exec = nullptr;
+    cudaGraphExec_t chunk_exec = nullptr;
     struct GraphGuard {
         cudaGraphExec_t* a;
-        cudaGraphExec_t* b;
         ~GraphGuard()
         {
             if (*a) cudaGraphExecDestroy(*a);
-            if (*b) cudaGraphExecDestroy(*b);
         }
-    } gguard{&chunk_exec, &rr_exec};
+    } gguard{&chunk_exec};
     auto capture_chunk = [&]() -> int {
         if (chunk_exec) {
             cudaGraphExecDestroy(chunk_exec);
@@ -2765,37 +2772,34 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         CK(cudaStreamSynchronize(s));
         return 0;
     };
-    // ---- Rayleigh-Ritz graph
-    {
-        cudaGraph_t graph;
-        CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-        launch_b_spmm(d_bp, np, rows, d_Q, d_T, 0, s);
-        launch_b_gram(d_bp, np, gram_b, maxm, d_Q, d_T, d_gpart, d_Aq, s);
-        if (hasB) {
-            launch_b_spmm(d_bp, np, rows, d_Q, d_T2, 1, s);
-            launch_b_gram(d_bp, np, gram_b, maxm, d_Q, d_T2, d_gpart, d_Bq, s);
-        } else {
-            launch_b_gram(d_bp, np, gram_b, maxm, d_Q, d_Q, d_gpart, d_Bq, s);
-        }
-        launch_b_reduced(d_bp, np, d_Aq, d_Bq, d_lam, d_Vr, d_mk, d_rwork, s);
-        launch_b_gemm(d_bp, np, gemm_b, d_Q, d_Vr, d_X, s);
-        launch_b_residual(d_bp, np, res_b, d_X, d_lam, d_Y, d_rpart, d_res, s);
-        CK(cudaStreamEndCapture(s, &graph));
-        cudaError_t e = cudaGraphInstantiate(&rr_exec, graph, 0);
-        cudaGraphDestroy(graph);
-        CK(e);
-    }
+    // ---- Rayleigh-Ritz step of the unfinished problems
+    auto rayleigh_ritz = [&]() -> int {
+        CK(launch_b_spmm(d_bp, np, rows, d_Q, d_T, 0, s));
+        CK(launch_b_gram(d_bp, np, gram_b, maxm, d_Q, d_T, d_gpart, d_Aq, s));
+        if (hasB) CK(launch_b_spmm(d_bp, np, rows, d_Q, d_T2, 1, s));
+        CK(launch_b_gram(d_bp, np, gram_b, maxm, d_Q, hasB ? d_T2 : d_Q, d_gpart, d_Bq, s));
+        CK(launch_b_reduced(d_bp, np, maxm, d_Aq, d_Bq, d_lam, d_Vr, d_mk, d_rwork, d_jwork, s));
+        CK(launch_b_gemm(d_bp, np, gemm_b, d_Q, d_Vr, d_X, s));
+        CK(launch_b_residual(d_bp, np, res_b, d_X, d_lam, d_Y, d_rpart, d_res, s));
+        return 0;
+    };
     // ---- refinement loops
+    std::vector<char> jwork(jacobi_batch_bytes(np));
     std::vector<double> lam(lo), res(lo), trace_prev(np, 0.0);
     std::vector<int> mk(np), maxres_ok(np, 0);
     long long total_steps = 0;
     int k = 0;
     for (k = 0;; ++k) {
-        CK(cudaGraphLaunch(rr_exec, s));
+        { const int rr = rayleigh_ritz(); if (rr) return rr; }
+        CK(cudaMemcpyAsync(jwork.data(), d_jwork, jwork.size(), cudaMemcpyDeviceToHost, s));
         CK(cudaMemcpyAsync(lam.data(), d_lam, sizeof(double) * lo, cudaMemcpyDeviceToHost, s));
         CK(cudaMemcpyAsync(res.data(), d_res, sizeof(double) * lo, cudaMemcpyDeviceToHost, s));
         CK(cudaMemcpyAsync(mk.data(), d_mk, sizeof(int) * np, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
+        if (jacobi_batch_failed(jwork.data(), np)) {
+            g_err = "reduced eigensolver: a wait exceeded the wait limit";
+            return -4;
+        }
         int left = 0;
         for (int p = 0; p < np; ++p) {
             if (done[p]) continue;

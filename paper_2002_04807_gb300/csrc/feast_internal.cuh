@@ -300,8 +300,14 @@ cudaError_t launch_b_gemm(const BProb* pr, int np, int nblocks, const double* A,
                           cudaStream_t s);
 cudaError_t launch_b_residual(const BProb* pr, int np, int nblocks, const double* X, const double* lam, double* R,
                               double* part, double* res, cudaStream_t s);
-cudaError_t launch_b_reduced(const BProb* pr, int np, const double* Aq, const double* Bq, double* lam, double* V,
-                             int* mk, double* work, cudaStream_t s);
+cudaError_t launch_b_reduced(const BProb* pr, int np, int maxm, const double* Aq, const double* Bq, double* lam, double* V,
+                             int* mk, double* work, void* jwork, cudaStream_t s);
+// Jacobi of every active problem's C (work area of b_reduce_prep) by teams of
+// CTAs: lam ascending, sorted eigenvectors in the area's third matrix (k_eig.cu).
+// work: jacobi_batch_bytes(np); jacobi_batch_failed looks at a host copy of it.
+size_t jacobi_batch_bytes(int np);
+cudaError_t launch_jacobi_batch(const BProb* pr, int np, int maxm, double* lam, double* bwork, void* work, cudaStream_t s);
+int jacobi_batch_failed(const void* host_work, int np);
 
 int num_sms();
 // kernel launches issued by this library (all threads), for launch accounting

@@ -18,6 +18,8 @@
 //   b_reduced     the reduced generalized eigenproblem of one problem per CTA
 //                 (m <= 128): two cyclic Jacobi decompositions in shared and
 //                 global memory, rounds synchronised with __syncthreads
+#include <algorithm>
+
 #include "chol.cuh"
 #include "feast_internal.cuh"
 
@@ -78,8 +80,11 @@ __device__ __forceinline__ void bdmma(double& c0, double& c1, double a, double b
                  : "d"(a), "d"(b));
 }
 
+// One BK step of a warp's 32 x 32 quarter; ni, nj: its 8 x 8 fragments in use
+// (the others lie outside the matrix), lo: fragments (i, j < i + lo) lie below
+// the diagonal of a symmetric result and are left out.
 __device__ __forceinline__ void btile_mma(const double (*As)[BLD], const double (*Bs)[BLD], double (&acc)[4][4][2],
-                                          int wr, int wc, int lane)
+                                          int wr, int wc, int lane, int ni, int nj, int lo)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -92,7 +97,8 @@ __device__ __forceinline__ void btile_mma(const double (*As)[BLD], const double 
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) bdmma(acc[i][j][0], acc[i][j][1], a[i], b[j]);
+            for (int j = 0; j < 4; ++j)
+                if (i < ni && j < nj && j >= i + lo) bdmma(acc[i][j][0], acc[i][j][1], a[i], b[j]);
     }
 }
 
@@ -125,6 +131,8 @@ __global__ void __launch_bounds__(128) b_gram(const BProb* pr, int np, int nbloc
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+    const int ni = min(4, max(0, (m - a0 - wr + 7) / 8)), nj = min(4, max(0, (m - b0 - wc + 7) / 8));
+    const int lo = ta == tb ? (wr - wc) / 8 : -4;
     for (int k0 = r0; k0 < r1; k0 += BK) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -136,7 +144,7 @@ __global__ void __launch_bounds__(128) b_gram(const BProb* pr, int np, int nbloc
             Bs[kk][c] = (rok && b0 + c < m) ? __ldg(Yp + (size_t)r * m + b0 + c) : 0.0;
         }
         __syncthreads();
-        btile_mma(As, Bs, acc, wr, wc, lane);
+        btile_mma(As, Bs, acc, wr, wc, lane, ni, nj, lo);
         __syncthreads();
     }
     double* out = part + P.gpart_off + (size_t)split * m * m;
@@ -161,21 +169,10 @@ __global__ void b_gram_reduce(const BProb* pr, const double* __restrict__ part, 
     const double* pp = part + P.gpart_off;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < m * m; idx += gridDim.x * blockDim.x) {
         const int i = idx / m, j = idx % m;
-        const int ti = i / BT, tj = j / BT;
-        double v;
-        if (ti == tj) {
-            double s1 = 0.0, s2 = 0.0;
-            for (int s = 0; s < ks; ++s) {
-                s1 += pp[(size_t)s * m * m + (size_t)i * m + j];
-                s2 += pp[(size_t)s * m * m + (size_t)j * m + i];
-            }
-            v = 0.5 * (s1 + s2);
-        } else {
-            const int a = ti < tj ? i : j, b = ti < tj ? j : i;
-            double s1 = 0.0;
-            for (int s = 0; s < ks; ++s) s1 += pp[(size_t)s * m * m + (size_t)a * m + b];
-            v = s1;
-        }
+        // the entry on or above the diagonal, mirrored
+        const int a = i < j ? i : j, b = i < j ? j : i;
+        double v = 0.0;
+        for (int s = 0; s < ks; ++s) v += pp[(size_t)s * m * m + (size_t)a * m + b];
         C[P.c_off + idx] = v;
     }
 }
@@ -205,6 +202,7 @@ __global__ void __launch_bounds__(128) b_gemm(const BProb* pr, int np, int nbloc
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+    const int ni = min(4, max(0, (n - r0 - wr + 7) / 8)), nj = min(4, max(0, (m - c0 - wc + 7) / 8));
     for (int k0 = 0; k0 < m; k0 += BK) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -217,7 +215,7 @@ __global__ void __launch_bounds__(128) b_gemm(const BProb* pr, int np, int nbloc
             Bs[bk][bc] = (vk < m && vc < m) ? __ldg(Vp + (size_t)vk * m + vc) : 0.0;
         }
         __syncthreads();
-        btile_mma(As, Bs, acc, wr, wc, lane);
+        btile_mma(As, Bs, acc, wr, wc, lane, ni, nj, -4);
         __syncthreads();
     }
     const int g = lane >> 2, tq = lane & 3;
@@ -401,15 +399,15 @@ __device__ void cta_jacobi(int m, double* A, double* V, CtaRot& R)
     }
 }
 
-// Reduced generalized problem of one problem per CTA (m <= 128): scale by
-// D = diag(B_Q)^{-1/2}; S = D L^{-T} from B~ = L L^T when the Cholesky
-// factor is accepted, else Jacobi on B~, keep d > 1e-14 max d,
-// S = D U_k d_k^{-1/2} (sentinel on dropped directions); C = S^T A~ S,
-// Jacobi on C, V = S W; lam
-// ascending (live values first), mk live count.  work: 6 m*m + 4 m doubles.
-__global__ void __launch_bounds__(kRedThreads) b_reduced(const BProb* pr, const double* __restrict__ Aq,
-                                                          const double* __restrict__ Bq, double* __restrict__ lam,
-                                                          double* __restrict__ Vout, int* __restrict__ mk,
+// Reduced generalized problems up to their standard form, one problem per CTA
+// (m <= 128): scale by D = diag(B_Q)^{-1/2}; S = D L^{-T} from B~ = L L^T when
+// the Cholesky factor is accepted, else Jacobi on B~, keep d > 1e-14 max d,
+// S = D U_k d_k^{-1/2} (sentinel on dropped directions); C = S^T A~ S and the
+// live count mk.  work, per problem: six m x m matrices (A~, B~, U, S, C, W)
+// and 4 m doubles; jacobi_team (k_eig.cu) diagonalises C with several CTAs per
+// problem and b_reduce_vectors forms V = S W.
+__global__ void __launch_bounds__(kRedThreads) b_reduce_prep(const BProb* pr, const double* __restrict__ Aq,
+                                                          const double* __restrict__ Bq, int* __restrict__ mk,
                                                           double* __restrict__ work)
 {
     __shared__ CtaRot R;
@@ -423,8 +421,7 @@ __global__ void __launch_bounds__(kRedThreads) b_reduced(const BProb* pr, const 
     double* U = Bt + mm;
     double* S = U + mm;
     double* C = S + mm;
-    double* Wv = C + mm;
-    double* dsc = Wv + mm;
+    double* dsc = C + 2 * mm;
     double* d = dsc + m;
     const double* aq = Aq + P.c_off;
     const double* bq = Bq + P.c_off;
@@ -444,7 +441,7 @@ __global__ void __launch_bounds__(kRedThreads) b_reduced(const BProb* pr, const 
     if (chol) {  // S = D L^{-T}
         for (int idx = threadIdx.x; idx < (int)mm; idx += blockDim.x) {
             const int r = idx / m, c = idx % m;
-            S[idx] = c > r ? dsc[r] * U[idx] : (c == r ? dsc[r] * xd[r] : 0.0);
+            S[idx] = c > r ? dsc[r] * U[chol_inv_at(m, c, r)] : (c == r ? dsc[r] * xd[r] : 0.0);
         }
     } else {
         cta_jacobi(m, Bt, U, R);
@@ -486,27 +483,24 @@ __global__ void __launch_bounds__(kRedThreads) b_reduced(const BProb* pr, const 
             if (zero) C[c * m + c] = kSentinelB;
         }
     }
-    __syncthreads();
-    cta_jacobi(m, C, Wv, R);
-    __syncthreads();
-    // V = S W with columns sorted by ascending eigenvalue
-    double* lp = lam + P.l_off;
-    double* vo = Vout + P.c_off;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        const double li = C[i * m + i];
-        int rank = 0;
-        for (int j = 0; j < m; ++j) {
-            const double lj = C[j * m + j];
-            rank += (lj < li) || (lj == li && j < i);
-        }
-        lp[rank] = li;
-        for (int r = 0; r < m; ++r) {
-            double s = 0.0;
-            for (int l = 0; l < m; ++l) s = fma(S[r * m + l], Wv[l * m + i], s);
-            vo[r * m + rank] = s;
-        }
-    }
     if (threadIdx.x == 0) mk[blockIdx.x] = live;
+}
+
+// V = S W (W sorted by jacobi_team); grid.y = problem
+__global__ void __launch_bounds__(256) b_reduce_vectors(const BProb* pr, const double* __restrict__ work, double* __restrict__ Vout)
+{
+    const BProb& P = pr[blockIdx.y];
+    if (!P.active) return;
+    const int m = P.m;
+    const size_t mm = (size_t)m * m;
+    const double* S = work + P.w_off + 3 * mm;
+    const double* W = work + P.w_off + 2 * mm;
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < (int)mm; idx += gridDim.x * blockDim.x) {
+        const int r = idx / m, c = idx % m;
+        double s = 0.0;
+        for (int l = 0; l < m; ++l) s = fma(__ldg(S + (size_t)r * m + l), __ldg(W + (size_t)l * m + c), s);
+        Vout[P.c_off + idx] = s;
+    }
 }
 
 // ---------------------------------------------------------------- launchers
@@ -552,11 +546,14 @@ cudaError_t launch_b_residual(const BProb* pr, int np, int nblocks, const double
     return cudaGetLastError();
 }
 
-cudaError_t launch_b_reduced(const BProb* pr, int np, const double* Aq, const double* Bq, double* lam, double* V,
-                             int* mk, double* work, cudaStream_t s)
+cudaError_t launch_b_reduced(const BProb* pr, int np, int maxm, const double* Aq, const double* Bq, double* lam, double* V,
+                             int* mk, double* work, void* jwork, cudaStream_t s)
 {
-    b_reduced<<<np, kRedThreads, 0, s>>>(pr, Aq, Bq, lam, V, mk, work);
-    count_launches(1);
+    b_reduce_prep<<<np, kRedThreads, 0, s>>>(pr, Aq, Bq, mk, work);
+    const cudaError_t e = launch_jacobi_batch(pr, np, maxm, lam, work, jwork, s);
+    if (e != cudaSuccess) return e;
+    b_reduce_vectors<<<dim3(std::max(1, maxm * maxm / 512), np), 256, 0, s>>>(pr, work, V);
+    count_launches(2);
     return cudaGetLastError();
 }
 

@@ -27,8 +27,11 @@
 // they sort last and the live count mk is the number of non-sentinel values.
 #include <atomic>
 
+#include <algorithm>
+
 #include "chol.cuh"
 #include "feast_internal.cuh"
+#include "team.cuh"
 
 namespace feast {
 
@@ -38,201 +41,290 @@ static constexpr int kEigThreads = 256;
 
 static constexpr int kMaxHalf = 4096;  // m <= 8192
 
-struct GridBar {
-    unsigned long long count;  // arrivals since launch; never reset
-    int err;
-    int pad;
-};
-
 struct JacWork {
-    GridBar bar;
-    double fro;
+    unsigned count;  // barrier arrivals
+    int err;
     int sweeps;
     int status;
+    int again[2];  // a sweep left an entry above the threshold
 };
 
-// Spin limit of the grid barrier in SM clock cycles (about two seconds at
+struct JacTask {
+    int m;
+    double *A, *A2, *V, *lam, *Vout;
+};
+struct JacArgs {
+    const BProb* pr;  // batch: the problems, their work areas and Ritz values
+    double *bwork, *blam;
+    JacTask one;
+    int ntask, nteams, nc;
+    JacWork* work;  // [nteams], zeroed
+    long long limit;
+};
+
+// Spin limit of the barriers in SM clock cycles (about two seconds at
 // 2 GHz); feast_set_wait_limit changes it for the launches that follow.
 static constexpr long long kDefaultSpinCycles = 4000000000LL;
 static std::atomic<long long> g_spin_cycles{kDefaultSpinCycles};
 long long wait_limit_cycles() { return g_spin_cycles.load(); }
 
-// Bounded grid barrier for a cooperative launch: each CTA adds one arrival to
-// a counter that only grows, then waits until the counter reaches the end of
-// its generation.  Returns false when any CTA spun longer than `limit` clock
-// cycles or an earlier barrier failed (the error flag is then set for all).
-__device__ __forceinline__ bool grid_sync(GridBar* b, long long limit)
-{
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int good = (*(volatile int*)&b->err == 0);
-        if (good) {
-            unsigned long long old;
-            asm volatile("atom.add.release.gpu.u64 %0, [%1], 1;" : "=l"(old) : "l"(&b->count) : "memory");
-            const unsigned long long target = (old / gridDim.x + 1) * gridDim.x;
-            const long long t0 = clock64();
-            for (;;) {
-                unsigned long long cur;
-                asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(cur) : "l"(&b->count) : "memory");
-                if (cur >= target) break;
-                if (*(volatile int*)&b->err) { good = 0; break; }
-                if (clock64() - t0 > limit) {
-                    atomicExch(&b->err, 1);
-                    good = 0;
-                    break;
-                }
-            }
-        }
-        ok = good;
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
 // round-robin partner table: slot 0 holds player 0, slot s >= 1 holds
 // player 1 + ((s - 1 + r) mod (mp - 1)); pair k is (slot k, slot mp-1-k)
 __device__ __forceinline__ int rr_player(int slot, int r, int mp)
 {
-    return slot == 0 ? 0 : 1 + (slot - 1 + r) % (mp - 1);
+    const int x = slot + r;  // r < mp - 1
+    return slot == 0 ? 0 : (x < mp ? x : x - (mp - 1));
 }
 
-// One grid barrier per round: every CTA computes all mp/2 rotations of the
-// round itself (identical inputs, identical code, so identical angles) into
-// shared memory, then updates its share of the 2x2 blocks from the current
-// copy of A into the other copy, so no CTA writes what another still reads.
+// Rotation of the pair (p, q): t near the smaller root of
+// f(t) = b t^2 + d t - b, b = apq, d = aqq - app (scaled near 1): the root in
+// single precision and one Newton step in FP64 (about 1e-13 of b is left), and
+// c = 1 / sqrt(1 + t^2), s = t c to FP64 (a single-precision seed and two
+// Newton steps), so the rotation is orthogonal to rounding although it leaves
+// -c^2 f(t) in the place of apq.  Fifteen FP64 operations instead of two
+// divisions and two square roots, which held every round up while all CTAs
+// computed all angles.
+__device__ __forceinline__ void jac_rotation(double d, double b, double& c, double& s, double& t)
+{
+    const float df = (float)d, bf = (float)b, h = 0.5f * df;
+    const float x = df == 0.0f ? 1.0f : copysignf(1.0f, h) * (bf / (fabsf(h) + sqrtf(fmaf(h, h, bf * bf))));
+    t = (double)x;
+    t = fma(-fma(fma(b, t, d), t, -b), (double)(1.0f / fmaf(2.0f * bf, x, df)), t);
+    const double y = fma(t, t, 1.0);
+    double r = (double)rsqrtf((float)y);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) r = r * fma(-0.5 * y * r, r, 1.5);
+    c = r;
+    s = t * r;
+}
+
+// Cyclic Jacobi of one matrix by a team of CTAs, one barrier per round: every
+// CTA computes all mp/2 rotations of the round itself (identical inputs and
+// code, so identical angles) into shared memory, then its share of the 2x2
+// blocks from the current copy of A into the other copy, so no CTA writes what
+// another still reads.  Of two blocks that mirror each other one is computed
+// and written twice.  A round is a chain of latencies (at m = 150 with 90 CTAs
+// 1.3 us of loads and angles, 1.2 the blocks, 0.4 V, 1.7 the barrier; FP64
+// operations take some 100 cycles one after the other): the entries of a
+// thread's first block and of its first pair of V load together with those of
+// the angles, and its place in the round's table is worked out once.  7.7 us a
+// round before, 4.6 now.  A sweep ends with a look for
+// entries above the threshold, so no whole sweep is spent on finding none.
 // Rotation tables in dynamic shared memory: c, s, t (doubles), p, q (ints).
-__global__ void __launch_bounds__(kEigThreads) jacobi_coop(int m, double* A, double* A2, double* V, double* lam,
-                                                          double* Vout, JacWork* w, long long limit)
+// Tasks: `one` (pr == nullptr) or the batch's active problems in turn.
+__global__ void __launch_bounds__(kEigThreads) jacobi_team(JacArgs a)
 {
     extern __shared__ double rsh[];
-    const int mp = m + (m & 1);
-    const int half = mp / 2;
-    double* rc = rsh;
-    double* rs = rc + half;
-    double* rt = rs + half;
-    int* rp = (int*)(rt + half);
-    int* rq = rp + half;
-    __shared__ int any;
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int gsz = gridDim.x * blockDim.x;
-    // V = I
-    for (long long idx = gtid; idx < (long long)m * m; idx += gsz) V[idx] = (idx / m == idx % m) ? 1.0 : 0.0;
-    if (blockIdx.x == 0) {
-        __shared__ double red[kEigThreads];
-        double s = 0.0;
+    __shared__ double sred[kEigThreads];
+    const int nc = a.nc, team = blockIdx.x / nc, cta = blockIdx.x - team * nc;
+    JacWork* w = a.work + team;
+    unsigned target = 0;
+    const int gtid = cta * blockDim.x + threadIdx.x, gsz = nc * blockDim.x;
+    for (int task = team; task < a.ntask; task += a.nteams) {
+        int m = a.one.m;
+        double *A = a.one.A, *A2 = a.one.A2, *V = a.one.V, *lam = a.one.lam, *Vout = a.one.Vout;
+        if (a.pr) {
+            const BProb& P = a.pr[task];
+            if (!P.active) continue;
+            m = P.m;
+            const size_t mm = (size_t)m * m;
+            double* W0 = a.bwork + P.w_off;  // layout of b_reduce_prep (k_batch.cu)
+            A = W0 + 4 * mm;
+            A2 = W0 + mm;
+            V = W0 + 5 * mm;
+            Vout = W0 + 2 * mm;
+            lam = a.blam + P.l_off;
+        }
+        const int mp = m + (m & 1), half = mp / 2;
+        double* rc = rsh;
+        double* rs = rc + half;
+        double* rt = rs + half;
+        int* rp = (int*)(rt + half);
+        int* rq = rp + half;
+        for (long long idx = gtid; idx < (long long)m * m; idx += gsz) V[idx] = (idx / m == idx % m) ? 1.0 : 0.0;
+        double fr = 0.0;  // every CTA sums the same entries in the same order
         for (long long idx = threadIdx.x; idx < (long long)m * m; idx += blockDim.x)
-            s += fabs(A[idx]) < 1e299 ? A[idx] * A[idx] : 0.0;  // sentinels excluded
-        red[threadIdx.x] = s;
+            fr += fabs(A[idx]) < 1e299 ? A[idx] * A[idx] : 0.0;  // sentinels excluded
+        sred[threadIdx.x] = fr;
         __syncthreads();
         for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+            if (threadIdx.x < o) sred[threadIdx.x] += sred[threadIdx.x + o];
             __syncthreads();
         }
-        if (threadIdx.x == 0) w->fro = sqrt(red[0]);
-    }
-    if (!grid_sync(&w->bar, limit)) return;
-    const double absfloor = 1e-18 * *(volatile double*)&w->fro;
-    double* cur = A;
-    double* nxt = A2;
-    int sweep = 0;
-    for (; sweep < kMaxSweeps && mp >= 2; ++sweep) {
-        if (threadIdx.x == 0) any = 0;
-        __syncthreads();
-        for (int r = 0; r < mp - 1; ++r) {
-            for (int k = threadIdx.x; k < half; k += blockDim.x) {
-                int p = rr_player(k, r, mp), q = rr_player(mp - 1 - k, r, mp);
-                if (p > q) { const int t = p; p = q; q = t; }
-                double c = 1.0, sn = 0.0, t = 0.0;
-                if (q < m) {
-                    const double apq = __ldcg(cur + (size_t)p * m + q);
-                    const double app = __ldcg(cur + (size_t)p * m + p), aqq = __ldcg(cur + (size_t)q * m + q);
-                    const double thr = fmax(1.1e-16 * sqrt(fabs(app * aqq)), absfloor);
-                    if (fabs(apq) > thr) {
-                        const double tau = (aqq - app) / (2.0 * apq);
-                        t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        c = 1.0 / sqrt(1.0 + t * t);
-                        sn = t * c;
-                        any = 1;
-                    }
-                }
-                rc[k] = c;
-                rs[k] = sn;
-                rt[k] = t;
-                rp[k] = p;
-                rq[k] = q;
+        const double fro = sqrt(sred[0]);
+        if (cta == 0 && threadIdx.x == 0) w->again[0] = w->again[1] = 0;
+        if (!team_sync(&w->count, target, nc, &w->err, a.limit)) return;
+        const double sc = fro > 0.0 && fro < 1e300 ? ldexp(1.0, -ilogb(fro)) : 1.0;
+        // |x| above 1.1e-16 sqrt(|xp xq|) and the floor of 1e-18 of the matrix, all
+        // scaled by sc: the norm is near 1, nothing under- or overflows
+        auto above = [](float x, float xp, float xq) {
+            return fabsf(x) > 1e-18f && x * x > 1.21e-32f * fabsf(xp) * fabsf(xq);
+        };
+        double* cur = A;
+        double* nxt = A2;
+        // every unordered pair of pairs {k, l} once, with no gaps inside a warp: row
+        // k, then l = k + 1, k + 2, ... around the circle; the diagonal blocks, whose
+        // arithmetic differs, after all the others
+        const int ncol = half / 2, nblk = half * (ncol + 1);
+        auto block = [&](int idx, int& k, int& l) {
+            if (idx >= half * ncol) {
+                k = l = idx - half * ncol;
+                return idx < nblk;
             }
-            __syncthreads();
-            // 2x2 block (k, l): rows of pair k, columns of pair l, cur -> nxt
-            for (long long idx = gtid; idx < (long long)half * half; idx += gsz) {
-                const int k = (int)(idx / half), l = (int)(idx % half);
-                const int p = rp[k], q = rq[k], pp = rp[l], qq = rq[l];
-                const bool qv = q < m, qqv = qq < m;
-                if (k == l) {  // diagonal block: closed form
-                    const double app = __ldcg(cur + (size_t)p * m + p);
-                    if (!qv) {
-                        nxt[(size_t)p * m + p] = app;
+            k = idx / ncol;
+            const int d = idx - k * ncol + 1;
+            l = k + d < half ? k + d : k + d - half;
+            return 2 * d < half || k < half / 2;
+        };
+        auto pair = [&](int k, int r, int& p, int& q) {
+            p = rr_player(k, r, mp);
+            q = rr_player(mp - 1 - k, r, mp);
+            if (p > q) {
+                const int t = p;
+                p = q;
+                q = t;
+            }
+        };
+        // a thread's first block (k, l) and first pair of a row of V
+        int k0 = 0, l0 = 0;
+        const bool has = block(gtid, k0, l0), hasv = gtid < m * half;
+        const int i0 = gtid / half, kv0 = gtid - i0 * half;
+        int sweep = 0;
+        for (; sweep < kMaxSweeps && mp >= 2; ++sweep) {
+            for (int r = 0; r < mp - 1; ++r) {
+                double x00 = 0.0, x01 = 0.0, x10 = 0.0, x11 = 0.0, vp = 0.0, vq = 0.0;
+                auto load = [&](int p, int q, int pp, int qq) {
+                    x00 = __ldcg(cur + (size_t)p * m + pp);
+                    x01 = qq < m ? __ldcg(cur + (size_t)p * m + qq) : 0.0;
+                    x10 = q < m ? __ldcg(cur + (size_t)q * m + pp) : 0.0;
+                    x11 = q < m && qq < m ? __ldcg(cur + (size_t)q * m + qq) : 0.0;
+                };
+                if (has) {
+                    int p, q, pp, qq;
+                    pair(k0, r, p, q);
+                    pair(l0, r, pp, qq);
+                    load(p, q, pp, qq);
+                }
+                if (hasv) {
+                    int p, q;
+                    pair(kv0, r, p, q);
+                    vp = __ldcg(V + (size_t)i0 * m + p);
+                    vq = q < m ? __ldcg(V + (size_t)i0 * m + q) : 0.0;
+                }
+                for (int k = threadIdx.x; k < half; k += blockDim.x) {
+                    int p, q;
+                    pair(k, r, p, q);
+                    double c = 1.0, sn = 0.0, t = 0.0;
+                    if (q < m) {
+                        const double apq = __ldcg(cur + (size_t)p * m + q);
+                        const double app = __ldcg(cur + (size_t)p * m + p), aqq = __ldcg(cur + (size_t)q * m + q);
+                        const double b = apq * sc, xp = app * sc, xq = aqq * sc;
+                        if (above((float)b, (float)xp, (float)xq)) jac_rotation(xq - xp, b, c, sn, t);
+                    }
+                    rc[k] = c;
+                    rs[k] = sn;
+                    rt[k] = t;
+                    rp[k] = p;
+                    rq[k] = q;
+                }
+                __syncthreads();
+                for (int idx = gtid; idx < nblk; idx += gsz) {
+                    int k = k0, l = l0;
+                    if (idx == gtid ? !has : !block(idx, k, l)) continue;
+                    const int p = rp[k], q = rq[k], pp = rp[l], qq = rq[l];
+                    const bool qv = q < m, qqv = qq < m;
+                    if (idx != gtid) load(p, q, pp, qq);
+                    if (k == l) {
+                        // diagonal block, with f(t): app - t apq + c^2 t f, aqq + t apq - c^2 t f, -c^2 f
+                        const double t = rt[k];
+                        const double e = rc[k] * rc[k] * fma(fma(x01, t, x11 - x00), t, -x01);
+                        const double ta = fma(-t, e, t * x01);
+                        nxt[(size_t)p * m + p] = x00 - ta;
+                        if (qv) {
+                            nxt[(size_t)q * m + q] = x11 + ta;
+                            nxt[(size_t)p * m + q] = nxt[(size_t)q * m + p] = -e;
+                        }
                         continue;
                     }
-                    const double apq = __ldcg(cur + (size_t)p * m + q), aqq = __ldcg(cur + (size_t)q * m + q);
-                    if (rs[k] == 0.0) {
-                        nxt[(size_t)p * m + p] = app;
-                        nxt[(size_t)q * m + q] = aqq;
-                        nxt[(size_t)p * m + q] = apq;
-                        nxt[(size_t)q * m + p] = __ldcg(cur + (size_t)q * m + p);
-                    } else {
-                        nxt[(size_t)p * m + p] = app - rt[k] * apq;
-                        nxt[(size_t)q * m + q] = aqq + rt[k] * apq;
-                        nxt[(size_t)p * m + q] = 0.0;
-                        nxt[(size_t)q * m + p] = 0.0;
+                    const double ck = rc[k], sk = rs[k], cl = rc[l], sl = rs[l];
+                    // rows: new row p = c row p - s row q ; new row q = s row p + c row q
+                    const double y00 = ck * x00 - sk * x10, y01 = ck * x01 - sk * x11;
+                    const double y10 = sk * x00 + ck * x10, y11 = sk * x01 + ck * x11;
+                    // columns: new col p' = c col p' - s col q' ; new col q' = s col p' + c col q'
+                    const double z00 = cl * y00 - sl * y01, z01 = sl * y00 + cl * y01;
+                    const double z10 = cl * y10 - sl * y11, z11 = sl * y10 + cl * y11;
+                    nxt[(size_t)p * m + pp] = z00;
+                    nxt[(size_t)pp * m + p] = z00;
+                    if (qqv) {
+                        nxt[(size_t)p * m + qq] = z01;
+                        nxt[(size_t)qq * m + p] = z01;
                     }
-                    continue;
+                    if (qv) {
+                        nxt[(size_t)q * m + pp] = z10;
+                        nxt[(size_t)pp * m + q] = z10;
+                    }
+                    if (qv && qqv) {
+                        nxt[(size_t)q * m + qq] = z11;
+                        nxt[(size_t)qq * m + q] = z11;
+                    }
                 }
-                const double ck = rc[k], sk = rs[k], cl = rc[l], sl = rs[l];
-                const double x00 = __ldcg(cur + (size_t)p * m + pp);
-                const double x01 = qqv ? __ldcg(cur + (size_t)p * m + qq) : 0.0;
-                const double x10 = qv ? __ldcg(cur + (size_t)q * m + pp) : 0.0;
-                const double x11 = (qv && qqv) ? __ldcg(cur + (size_t)q * m + qq) : 0.0;
-                // rows: new row p = c row p - s row q ; new row q = s row p + c row q
-                const double y00 = ck * x00 - sk * x10, y01 = ck * x01 - sk * x11;
-                const double y10 = sk * x00 + ck * x10, y11 = sk * x01 + ck * x11;
-                // columns: new col p' = c col p' - s col q' ; new col q' = s col p' + c col q'
-                nxt[(size_t)p * m + pp] = cl * y00 - sl * y01;
-                if (qqv) nxt[(size_t)p * m + qq] = sl * y00 + cl * y01;
-                if (qv) nxt[(size_t)q * m + pp] = cl * y10 - sl * y11;
-                if (qv && qqv) nxt[(size_t)q * m + qq] = sl * y10 + cl * y11;
+                for (int idx = gtid; idx < m * half; idx += gsz) {
+                    const int i = idx == gtid ? i0 : idx / half, k = idx == gtid ? kv0 : idx - i * half;
+                    const double sk = rs[k];
+                    if (sk == 0.0) continue;
+                    const double ck = rc[k];
+                    const int p = rp[k], q = rq[k];
+                    if (idx != gtid) {
+                        vp = __ldcg(V + (size_t)i * m + p);
+                        vq = __ldcg(V + (size_t)i * m + q);
+                    }
+                    V[(size_t)i * m + p] = ck * vp - sk * vq;
+                    V[(size_t)i * m + q] = sk * vp + ck * vq;
+                }
+                if (!team_sync(&w->count, target, nc, &w->err, a.limit)) return;
+                double* tmp = cur;
+                cur = nxt;
+                nxt = tmp;
             }
-            for (long long idx = gtid; idx < (long long)m * half; idx += gsz) {
-                const int i = (int)(idx / half), k = (int)(idx % half);
-                const double sk = rs[k];
-                if (sk == 0.0) continue;
-                const double ck = rc[k];
-                const int p = rp[k], q = rq[k];
-                const double vp = V[(size_t)i * m + p], vq = V[(size_t)i * m + q];
-                V[(size_t)i * m + p] = ck * vp - sk * vq;
-                V[(size_t)i * m + q] = sk * vp + ck * vq;
+            // entries still above the threshold?
+            int more = 0;
+            for (int idx = gtid; idx < m * m; idx += gsz) {
+                const int i = idx / m, j = idx % m;
+                if (j <= i) continue;
+                const double x = __ldcg(cur + idx);
+                if (above((float)(x * sc), (float)(__ldcg(cur + (size_t)i * m + i) * sc), (float)(__ldcg(cur + (size_t)j * m + j) * sc)))
+                    more = 1;
             }
-            if (!grid_sync(&w->bar, limit)) return;
-            double* tmp = cur;
-            cur = nxt;
-            nxt = tmp;
+            if (__syncthreads_or(more) && threadIdx.x == 0) w->again[sweep & 1] = 1;
+            if (!team_sync(&w->count, target, nc, &w->err, a.limit)) return;
+            const int go = *(volatile int*)&w->again[sweep & 1];
+            if (!go) break;  // same decision in every CTA
+            // the other flag is read next; nobody reads it before the next barrier
+            if (cta == 0 && threadIdx.x == 0) *(volatile int*)&w->again[(sweep & 1) ^ 1] = 0;
         }
-        if (!any) break;  // same decision in every CTA
-    }
-    // ascending order: rank of each diagonal entry (ties by index)
-    for (int i = gtid; i < m; i += gsz) {
-        const double li = __ldcg(cur + (size_t)i * m + i);
-        int rank = 0;
-        for (int j = 0; j < m; ++j) {
-            const double lj = __ldcg(cur + (size_t)j * m + j);
-            rank += (lj < li) || (lj == li && j < i);
+        // ascending order: rank of each diagonal entry (ties by index)
+        double* dg = rsh;  // rotation tables are free: m doubles and m ranks fit
+        int* rank = (int*)(dg + mp);
+        __syncthreads();
+        for (int i = threadIdx.x; i < m; i += blockDim.x) dg[i] = __ldcg(cur + (size_t)i * m + i);
+        __syncthreads();
+        for (int i = threadIdx.x; i < m; i += blockDim.x) {
+            const double li = dg[i];
+            int k = 0;
+            for (int j = 0; j < m; ++j) k += (dg[j] < li) || (dg[j] == li && j < i);
+            rank[i] = k;
+            if (cta == 0) lam[k] = li;
         }
-        lam[rank] = li;
-        for (int row = 0; row < m; ++row) Vout[(size_t)row * m + rank] = V[(size_t)row * m + i];
-    }
-    if (gtid == 0) {
-        w->sweeps = sweep;
-        w->status = sweep >= kMaxSweeps ? -1 : 0;
+        __syncthreads();
+        for (long long idx = gtid; idx < (long long)m * m; idx += gsz) {
+            const int row = (int)(idx / m), i = (int)(idx % m);
+            Vout[(size_t)row * m + rank[i]] = __ldcg(V + idx);
+        }
+        if (gtid == 0) {
+            w->sweeps = sweep;
+            w->status = sweep >= kMaxSweeps ? -1 : 0;
+        }
+        __syncthreads();
     }
 }
 
@@ -247,22 +339,50 @@ size_t jacobi_work_bytes(int m)
     return 1024 + sizeof(JacWork) + 2 * sizeof(double) * (size_t)m * m;
 }
 
-static int coop_grid(int m)
+// CTAs of a team, within `most`.
+static int jacobi_ctas(int m, int most)
 {
-    static const int per_sm = [] {  // initialised once, thread-safe
-        int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, jacobi_coop, kEigThreads, rot_smem(2 * kMaxHalf));
-        return v > 0 ? v : 1;
-    }();
-    const int mp = m + (m & 1);
-    const long long work = (long long)m * (mp / 2) > (long long)(mp / 2) * (mp / 2) ? (long long)m * (mp / 2)
-                                                                                    : (long long)(mp / 2) * (mp / 2);
-    long long blocks = (work + kEigThreads - 1) / kEigThreads;
-    const long long cap = (long long)num_sms() * per_sm;
-    if (blocks > cap) blocks = cap;
-    if (blocks > num_sms()) blocks = num_sms();
-    if (blocks < 1) blocks = 1;
-    return (int)blocks;
+    // a warp instruction holds the FP64 pipe for 16 cycles, so the blocks are
+    // spread until a CTA has few warps of them
+    const long long half = (m + 1) / 2, work = half * (half / 2 + 1);
+    return (int)std::max(1LL, std::min<long long>((work + 31) / 32, most));
+}
+
+static cudaError_t launch_jacobi(JacArgs a, int m, cudaStream_t s)
+{
+    const size_t smem = rot_smem(m);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(jacobi_team, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    a.limit = wait_limit_cycles();
+    void* args[] = {&a};
+    count_launches(1);
+    return cudaLaunchCooperativeKernel((void*)jacobi_team, dim3(a.nteams * a.nc), dim3(kEigThreads), args, smem, s);
+}
+
+size_t jacobi_batch_bytes(int np) { return sizeof(JacWork) * (size_t)std::min(np, num_sms()); }
+
+cudaError_t launch_jacobi_batch(const BProb* pr, int np, int maxm, double* lam, double* bwork, void* work, cudaStream_t s)
+{
+    JacArgs a = {};
+    a.pr = pr;
+    a.ntask = np;
+    a.nteams = std::min(np, num_sms());
+    a.nc = jacobi_ctas(maxm, num_sms() / a.nteams);
+    a.blam = lam;
+    a.bwork = bwork;
+    a.work = (JacWork*)work;
+    const cudaError_t e = cudaMemsetAsync(work, 0, sizeof(JacWork) * a.nteams, s);
+    return e != cudaSuccess ? e : launch_jacobi(a, maxm, s);
+}
+
+int jacobi_batch_failed(const void* host_work, int np)
+{
+    const JacWork* w = (const JacWork*)host_work;
+    for (int t = 0; t < std::min(np, num_sms()); ++t)
+        if (w[t].err) return 1;
+    return 0;
 }
 
 static char* align256(char* p) { return (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255); }
@@ -280,25 +400,61 @@ int jacobi_eig_dev(int m, double* A, double* lam, double* V, void* work, cudaStr
     p = align256(p + sizeof(double) * (size_t)m * m);
     double* Vw = (double*)p;
     if (cudaMemsetAsync(w, 0, sizeof(JacWork), s) != cudaSuccess) return -3;
-    const size_t smem = rot_smem(m);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(jacobi_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return -3;
-    int grid = coop_grid(m);
-    long long limit = g_spin_cycles.load();
-    void* args[] = {&m, &A, &A2, &Vw, &lam, &V, &w, &limit};
-    cudaError_t e = cudaLaunchCooperativeKernel((void*)jacobi_coop, dim3(grid), dim3(kEigThreads), args, smem, s);
-    count_launches(1);
-    if (e != cudaSuccess) return -3;
+    JacArgs a = {};
+    a.ntask = a.nteams = 1;
+    a.nc = jacobi_ctas(m, num_sms());
+    a.one = {m, A, A2, Vw, lam, V};
+    a.work = w;
+    if (launch_jacobi(a, m, s) != cudaSuccess) return -3;
     if (sweeps_host) {
         JacWork h;
         if (cudaMemcpyAsync(&h, w, sizeof(JacWork), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -3;
         if (cudaStreamSynchronize(s) != cudaSuccess) return -3;
         *sweeps_host = h.sweeps;
-        if (h.bar.err) return -2;
+        if (h.err) return -2;
         if (h.status) return -1;
     }
     return 0;
+}
+
+// ---------------------------------------------------------------- products of the reduced matrices
+// C = A B (TA = 0) or A^T B with C symmetric, its part on and above the diagonal
+// mirrored (TA = 1); all m x m.  A thread per element, 16 x 16 tiles: about
+// (m / 16)^2 CTAs, where the 64 x 64 tiles of the n x m products would leave
+// most of the chip idle (m = 150: 200 us, here 14).
+template <int TA>
+__global__ void __launch_bounds__(256) rg_product(int m, const double* __restrict__ A, const double* __restrict__ B,
+                                                  double* __restrict__ C)
+{
+    __shared__ double sa[16][17], sb[16][17];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int i0 = blockIdx.y * 16, j0 = blockIdx.x * 16;
+    if (TA && j0 < i0) return;
+    double s = 0.0;
+    for (int k0 = 0; k0 < m; k0 += 16) {
+        const int ai = TA ? k0 + ty : i0 + ty, aj = TA ? i0 + tx : k0 + tx;
+        const double av = ai < m && aj < m ? __ldg(A + (size_t)ai * m + aj) : 0.0;
+        if (TA) sa[tx][ty] = av;
+        else sa[ty][tx] = av;
+        sb[ty][tx] = k0 + ty < m && j0 + tx < m ? __ldg(B + (size_t)(k0 + ty) * m + j0 + tx) : 0.0;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 16; ++k) s = fma(sa[ty][k], sb[k][tx], s);
+        __syncthreads();
+    }
+    const int i = i0 + ty, j = j0 + tx;
+    if (i >= m || j >= m || (TA && j < i)) return;
+    C[(size_t)i * m + j] = s;
+    if (TA) C[(size_t)j * m + i] = s;
+}
+
+template <int TA>
+static cudaError_t launch_rg_product(int m, const double* A, const double* B, double* C, cudaStream_t s)
+{
+    const unsigned t = (unsigned)((m + 15) / 16);
+    rg_product<TA><<<dim3(t, t), 256, 0, s>>>(m, A, B, C);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- generalized problem
@@ -348,14 +504,14 @@ __global__ void rg_sentinel(int m, const double* S, double* C)
 // fit, else in the global scratch G; S = D X^T with X = L^{-1};
 // status = 0 when accepted (and *mk = m), 1 otherwise.
 static constexpr int kCholThreads = 1024;
-static constexpr size_t kCholSmemMax = 224 * 1024;
+static constexpr size_t kCholSmemMax = 216 * 1024;
 
 __global__ void __launch_bounds__(kCholThreads) rg_cholinv(int m, const double* __restrict__ Bt,
                                                            const double* __restrict__ dsc, double* __restrict__ S,
                                                            double* G, int use_smem, int* status, int* mk)
 {
     extern __shared__ double sh[];
-    __shared__ double red[kCholThreads / 32];
+    __shared__ double red[kCholThreads];
     double* M = use_smem ? sh : G;
     double* xd = M + (size_t)m * m;
     double* cj = xd + m;
@@ -365,7 +521,7 @@ __global__ void __launch_bounds__(kCholThreads) rg_cholinv(int m, const double* 
     if (ok) {
         for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
             const int r = idx / m, c = idx % m;
-            S[idx] = c > r ? dsc[r] * M[idx] : (c == r ? dsc[r] * xd[r] : 0.0);
+            S[idx] = c > r ? dsc[r] * M[chol_inv_at(m, c, r)] : (c == r ? dsc[r] * xd[r] : 0.0);
         }
     }
     if (threadIdx.x == 0) {
@@ -379,10 +535,7 @@ static size_t chol_bytes(int m) { return ((size_t)m * m + 2 * (size_t)m) * sizeo
 size_t reduced_work_bytes(int m)
 {
     const size_t mm = (size_t)m * m * sizeof(double);
-    int ks = 0;
-    const size_t gp = gram_partial_doubles(m, m, &ks, num_sms()) * sizeof(double);
-    return 8 * (mm + 256) + (m * sizeof(double) + 256) * 2 + gp + 256 + jacobi_work_bytes(m) + chol_bytes(m) +
-           512 + 1024;
+    return 8 * (mm + 256) + (m * sizeof(double) + 256) * 2 + jacobi_work_bytes(m) + chol_bytes(m) + 512 + 1024;
 }
 
 // lam[m] (ascending, sentinels >= 1e299 last), V row-major m x m, *mk (device).
@@ -405,9 +558,6 @@ int reduced_gev_dev(int m, const double* Aq, const double* Bq, double* lam, doub
     double* W = (double*)take(mm * 8);
     double* d = (double*)take(m * 8);
     double* dsc = (double*)take(m * 8);
-    int ks = 0;
-    const size_t gp = gram_partial_doubles(m, m, &ks, num_sms());
-    double* gpart = (double*)take(gp * 8);
     void* jw = take(jacobi_work_bytes(m));
     double* G = (double*)take(chol_bytes(m));
     int* cst = (int*)take(256);
@@ -425,11 +575,11 @@ int reduced_gev_dev(int m, const double* Aq, const double* Bq, double* lam, doub
     if (cudaMemcpyAsync(&hst, cst, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -4;
     if (cudaStreamSynchronize(s) != cudaSuccess) return -4;
     if (hst == 0) {
-        if (launch_gemm_nn_f64(m, m, m, At, S, T1, s) != cudaSuccess) return -4;
-        if (launch_gram_f64(m, m, S, T1, C, gpart, ks, 1, s) != cudaSuccess) return -4;
+        if (launch_rg_product<0>(m, At, S, T1, s) != cudaSuccess) return -4;
+        if (launch_rg_product<1>(m, S, T1, C, s) != cudaSuccess) return -4;
         const int st = jacobi_eig_dev(m, C, lam, W, jw, s, &sweeps);
         if (st) return st == -3 ? -4 : -3;
-        if (launch_gemm_nn_f64(m, m, m, S, W, V, s) != cudaSuccess) return -4;
+        if (launch_rg_product<0>(m, S, W, V, s) != cudaSuccess) return -4;
         return 0;
     }
     count_launches(2);  // basis, sentinel
@@ -437,13 +587,13 @@ int reduced_gev_dev(int m, const double* Aq, const double* Bq, double* lam, doub
     if (st) return st == -3 ? -4 : -3;
     rg_basis<<<blocks, 256, 0, s>>>(m, d, U, dsc, S, mk);
     if (cudaGetLastError() != cudaSuccess) return -4;
-    if (launch_gemm_nn_f64(m, m, m, At, S, T1, s) != cudaSuccess) return -4;
-    if (launch_gram_f64(m, m, S, T1, C, gpart, ks, 1, s) != cudaSuccess) return -4;
+    if (launch_rg_product<0>(m, At, S, T1, s) != cudaSuccess) return -4;
+    if (launch_rg_product<1>(m, S, T1, C, s) != cudaSuccess) return -4;
     rg_sentinel<<<(m + 255) / 256, 256, 0, s>>>(m, S, C);
     if (cudaGetLastError() != cudaSuccess) return -4;
     st = jacobi_eig_dev(m, C, lam, W, jw, s, &sweeps);
     if (st) return st == -3 ? -4 : -3;
-    if (launch_gemm_nn_f64(m, m, m, S, W, V, s) != cudaSuccess) return -4;
+    if (launch_rg_product<0>(m, S, W, V, s) != cudaSuccess) return -4;
     return 0;
 }
 
