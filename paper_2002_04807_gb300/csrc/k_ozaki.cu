@@ -7,21 +7,27 @@
 // and Rump ("Error-free transformations of matrix multiplication by using
 // fast routines of matrix multiplication", 2012):
 //   * every column c of X (of Y) gets a power of two 2^E_c > max_i |X[i][c]|;
-//   * |X[i][c]| 2^-E_c lies in [0, 1) and is written with kSlices base-2^7
-//     digits, |x| 2^-E = sum_s d_s 2^(-7 s) + r, d_s in [0, 127] (with the
-//     sign of x), 0 <= r < 2^(-7 kSlices); the digits come from the FP64 bit
-//     pattern by integer shifts and are exact in BF16;
-//   * X[i][a] Y[i][b] = 2^(E_a + F_b) sum_{s,t} d_s(i,a) e_t(i,b) 2^(-7 (s+t)),
-//     the pairs with s + t <= kSlices + 1 are kept (the rest weigh below
-//     2^(-7 kSlices) relative to 2^(E_a + F_b));
-//   * a level L = s + t has at most kSlices pairs of products below 2^14, so
-//     its sum over 128 rows stays below 2^24 and mma.sync accumulates it in
+//   * X[i][c] 2^-E_c is rounded to F 2^-55, F a signed integer of at most 2^55,
+//     and F is written with kSlices balanced base-2^8 digits, so that
+//     x 2^-E = sum_s d_s 2^(1 - 8 s) + r, d_s in [-128, 128], |r| <= 2^-56; the
+//     digits are the bytes of F plus a bias and are exact in BF16;
+//   * X[i][a] Y[i][b] = 2^(E_a + F_b) sum_{s,t} d_s(i,a) e_t(i,b) 2^(2 - 8 (s+t)),
+//     the pairs with s + t <= kSlices + 1 are kept (28; the rest weigh below
+//     2^(-53) relative to 2^(E_a + F_b) even with every digit at its largest);
+//   * a level L = s + t has at most kSlices pairs of products of at most 2^14,
+//     so its sum over 128 rows stays below 2^24 and mma.sync accumulates it in
 //     FP32 without any rounding; every 128 rows the level sums are folded,
 //     exactly, into two 64-bit integer accumulators (oz_fold), and at the end
 //     they are turned into FP64 once and the column scales 2^(E_a + F_b) are
 //     applied.
-// With kSlices = 8 the kept part is exact and the truncation error of an
+// With kSlices = 7 the kept part is exact and the truncation error of an
 // element is below 2^-55 |2^E_a| |2^F_b| per row: at FP64 level.
+// Eight 7-bit digits of |x| (36 pairs) gave the same error; cutting them took
+// 60 integer instructions a value and the ALU was the busiest unit (60 %, tensor
+// pipe 34 %: 1.31 ms at n = 262,144, m = 150).  A byte becomes a digit by one
+// byte permute into 2^23 + byte, one single-precision subtraction (a pipe that
+// is otherwise idle) and half a conversion: 1.00 ms, tensor pipe 35 %, ALU 49 %,
+// 51 % of the issue slots with three warps a scheduler.
 //
 // Layout: X, Y row-major n x m FP64.  A CTA (four warps) owns one 32 x 32
 // output tile of the upper tile triangle and a range of rows (split-K); each
@@ -42,7 +48,7 @@
 
 namespace feast {
 
-static constexpr int kSlices = 8;
+static constexpr int kSlices = 7;
 static constexpr int kOzTile = 32;                  // output tile side (CTA)
 static constexpr int kOzChunk = 32;                 // rows per shared-memory chunk
 static constexpr int kOzFlushChunks = 4;            // chunks per FP32 -> FP64 flush (128 rows)
@@ -71,51 +77,95 @@ __global__ void __launch_bounds__(256) oz_colexp(int n, int m, const double* __r
 // 2^-E_c is a normal double.
 __device__ __forceinline__ int oz_scale_exp(int field) { return min(max(field - 1022, -1022), 1022); }
 
-// The kSlices base-2^7 digits of |x| 2^-E, most significant first, with the
-// sign of x, by integer operations on the FP64 bit pattern (GB300's FP64 ALU
-// is too slow for the cut): |x| = M 2^(e - 1075) with M the 53-bit
-// significand, and F = floor(|x| 2^(56 - E)) = M 2^(e - 1075 - E + 56) < 2^56
-// because |x| < 2^E; then |x| 2^-E = sum_s d_s 2^(-7 (s + 1)) + r with
-// 0 <= r < 2^-56, d_s in [0, 127].
-__device__ __forceinline__ void oz_cut(double x, int E, float (&d)[kSlices])
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int ef = (int)((b >> 52) & 0x7ff);
-    const unsigned long long M = (b & 0xFFFFFFFFFFFFFull) | (ef ? (1ull << 52) : 0ull);
-    const int sh = (ef ? ef : 1) - 1075 - E + 56;  // <= 3 for |x| < 2^E
-    const unsigned long long F = sh >= 0 ? (M << min(sh, 3)) : (sh > -64 ? (M >> -sh) : 0ull);
-    const float sg = (b >> 63) ? -1.f : 1.f;
-#pragma unroll
-    for (int s = 0; s < kSlices; ++s) d[s] = sg * (float)(unsigned)((F >> (49 - 7 * s)) & 127ull);
-}
-
-// Exact folding of the FP32 level sums into two 64-bit integer accumulators.
-// Level l (weight 2^(-7 (l + 2))) holds an integer below 2^24, so
-//   hi = sum_{l < 4} P_l 2^(7 (3 - l))   in units of 2^-35,
-//   lo = sum_{l >= 4} P_l 2^(7 (7 - l))  in units of 2^-63,
-// are below 2^46 per flush and exact, and so are their running sums (below
-// 2^63 for up to 2^17 flushes).  FP64 (scarce on GB300) is used only once per
-// element at the end: value = hi 2^-35 + lo 2^-63.
-__device__ __forceinline__ void oz_fold(float (&P)[kSlices], long long& hi, long long& lo)
-{
-    long long h = 0, l = 0;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) h += (long long)__float2int_rn(P[s]) * (1LL << (7 * (3 - s)));
-#pragma unroll
-    for (int s = 4; s < kSlices; ++s) l += (long long)__float2int_rn(P[s]) * (1LL << (7 * (7 - s)));
-    hi += h;
-    lo += l;
-}
-
-__device__ __forceinline__ double oz_value(long long hi, long long lo, int e)
-{
-    return ldexp(fma((double)hi, 0x1p-35, (double)lo * 0x1p-63), e);
-}
-
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// F = x 2^(55 - E) rounded to an integer, plus the bias 0x80 in each of its
+// seven bytes: byte k is 128 + the digit of weight 2^(8 k), and the bits above
+// byte 5 are 128 + the leading digit (at most 256).  From the FP64 bit pattern
+// by integer operations (GB300's FP64 ALU is too slow for it): |x| = M 2^(e -
+// 1075), M < 2^53, so F = M 2^(e - 1020 - E) = (16 M / 2^t + 1) / 2 with
+// t = E + 1023 - e >= 0 (e = 1 for denormal numbers).
+__device__ __forceinline__ unsigned long long oz_fix(double x, int E)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int ef = (int)((hi >> 20) & 0x7ffu);
+    const unsigned mh = (hi & 0xFFFFFu) | (ef ? 0x100000u : 0u);
+    const unsigned long long M = (((unsigned long long)mh << 32) | lo) << 4;
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(M), "r"(E + 1023 - max(ef, 1)));  // amounts above 64 give 0
+    const unsigned long long F = (r + 1) >> 1;
+    const unsigned long long s = (unsigned long long)(long long)((int)hi >> 31);  // all ones when negative
+    return (F ^ s) + (0x80808080808080ull + (hi >> 31));
+}
+
+// The digits of two values (consecutive along the contraction), most
+// significant first, as BF16 pairs.
+__device__ __forceinline__ void oz_cut(double x0, double x1, int E0, int E1, uint32_t (&w)[kSlices])
+{
+    const unsigned long long G0 = oz_fix(x0, E0), G1 = oz_fix(x1, E1);
+    const unsigned a[2] = {(unsigned)G0, (unsigned)(G0 >> 32)}, b[2] = {(unsigned)G1, (unsigned)(G1 >> 32)};
+    constexpr float kBias = 8388608.0f + 128.0f;
+    w[0] = pack_bf16x2(__uint_as_float(0x4B000000u | (a[1] >> 16)) - kBias,
+                       __uint_as_float(0x4B000000u | (b[1] >> 16)) - kBias);
+#pragma unroll
+    for (int s = 1; s < kSlices; ++s) {
+        const int k = kSlices - 1 - s;  // byte
+        w[s] = pack_bf16x2(__uint_as_float(__byte_perm(a[k >> 2], 0x4B000000u, 0x7440 | (k & 3))) - kBias,
+                           __uint_as_float(__byte_perm(b[k >> 2], 0x4B000000u, 0x7440 | (k & 3))) - kBias);
+    }
+}
+
+// Exact folding of the FP32 level sums into two 64-bit integer accumulators.
+// Level l (weight 2^(-14 - 8 l)) holds an integer below 2^24, so
+//   hi = sum_{l < 3} P_l 2^(8 (2 - l))   in units of 2^-30,
+//   lo = sum_{l >= 3} P_l 2^(8 (6 - l))  in units of 2^-62,
+// are below 2^49 per flush and exact, and so are their running sums (below
+// 2^63 for up to 2^14 flushes, kOzMaxRows rows); value = hi 2^-30 + lo 2^-62.
+static constexpr long long kOzMaxRows = (1LL << 14) * 128;
+__device__ __forceinline__ void oz_fold(float (&P)[kSlices], long long& hi, long long& lo)
+{
+    long long h = 0, l = 0;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) h += (long long)__float2int_rn(P[s]) * (1LL << (8 * (2 - s)));
+#pragma unroll
+    for (int s = 3; s < kSlices; ++s) l += (long long)__float2int_rn(P[s]) * (1LL << (8 * (6 - s)));
+    hi += h;
+    lo += l;
+}
+
+// (hi 2^32 + lo) 2^(e - 62), rounded to nearest once, by integer operations:
+// two conversions, a product, an FMA and ldexp in FP64 held that pipe as long
+// as the tensor cores worked for an element of an n x 150 product.
+__device__ __forceinline__ double oz_value(long long hi, long long lo, int e)
+{
+    long long H = hi + (lo >> 32);
+    unsigned L = (unsigned)lo;
+    const bool neg = H < 0;
+    if (neg) {
+        H = -H - (L ? 1 : 0);
+        L = 0u - L;
+    }
+    unsigned long long N = (unsigned long long)H;
+    if (N == 0) return ldexp(neg ? -(double)L : (double)L, e - 62);
+    const int z = __clzll(H);
+    bool sticky = false;  // bits of L below N
+    if (z >= 32) {
+        N = (N << z) | ((unsigned long long)L << (z - 32));
+    } else {
+        N = (N << z) | (z ? L >> (32 - z) : 0u);
+        sticky = (L << z) != 0u;
+    }
+    const int ex = 1056 - z + e;  // biased exponent of the leading bit
+    unsigned long long m = N >> 11;
+    const unsigned r = (unsigned)N & 0x7ffu;
+    if (r > 0x400u || (r == 0x400u && (sticky || (m & 1)))) ++m;
+    if (ex <= 0 || ex >= 2046) return ldexp(neg ? -(double)m : (double)m, ex - 1075);
+    const unsigned long long bits = ((unsigned long long)(ex - 1) << 52) + m;
+    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
 }
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
@@ -208,16 +258,14 @@ __global__ void __launch_bounds__(kOzThreads, 3) gram_oz(int n, int m, const dou
         __syncthreads();  // the previous chunk's fragments have been read
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            float dx0[kSlices], dx1[kSlices], dy0[kSlices], dy1[kSlices];
-            oz_cut(vx[2 * u], Ex, dx0);
-            oz_cut(vx[2 * u + 1], Ex, dx1);
-            oz_cut(vy[2 * u], Ey, dy0);
-            oz_cut(vy[2 * u + 1], Ey, dy1);
+            uint32_t dx[kSlices], dy[kSlices];
+            oz_cut(vx[2 * u], vx[2 * u + 1], Ex, Ex, dx);
+            oz_cut(vy[2 * u], vy[2 * u + 1], Ey, Ey, dy);
             const int w = (warp + 4 * u) * kOzStride + lane;
 #pragma unroll
             for (int s = 0; s < kSlices; ++s) {
-                sA[s * kOzPlane + w] = pack_bf16x2(dx0[s], dx1[s]);
-                sB[s * kOzPlane + w] = pack_bf16x2(dy0[s], dy1[s]);
+                sA[s * kOzPlane + w] = dx[s];
+                sB[s * kOzPlane + w] = dy[s];
             }
         }
         __syncthreads();
@@ -289,6 +337,7 @@ size_t gram_oz_partial_doubles(int n, int m, int* ksplit_out, long long* rows_pe
     int ks = (3 * nsm) / tiles;  // one wave of three CTAs per SM
     const int maxk = (n + 255) / 256;        // at least 256 rows per split
     if (ks > maxk) ks = maxk;
+    ks = std::max(ks, (int)((n + kOzMaxRows - 1) / kOzMaxRows));  // the folds stay exact
     if (ks < 1) ks = 1;
     long long rps = ((long long)n + ks - 1) / ks;
     rps = (rps + kOzChunk - 1) / kOzChunk * kOzChunk;  // whole chunks
@@ -368,7 +417,7 @@ __global__ void oz_split_cols(int m, int k, int kp, int mp, const double* __rest
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
          t += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(t / half), j = (int)(t % half);
-        float d0[kSlices], d1[kSlices];
+        uint32_t d[kSlices];
         double v0 = 0.0, v1 = 0.0;
         int E = 0;
         if (c < k) {
@@ -376,10 +425,9 @@ __global__ void oz_split_cols(int m, int k, int kp, int mp, const double* __rest
             if (2 * j < m) v0 = V[(size_t)(2 * j) * k + c];
             if (2 * j + 1 < m) v1 = V[(size_t)(2 * j + 1) * k + c];
         }
-        oz_cut(v0, E, d0);
-        oz_cut(v1, E, d1);
+        oz_cut(v0, v1, E, E, d);
 #pragma unroll
-        for (int s = 0; s < kSlices; ++s) Vs[((size_t)s * kp + c) * half + j] = pack_bf16x2(d0[s], d1[s]);
+        for (int s = 0; s < kSlices; ++s) Vs[((size_t)s * kp + c) * half + j] = d[s];
     }
 }
 
@@ -435,11 +483,10 @@ __global__ void __launch_bounds__(kOzThreads, 3) gemm_oz(int n, int m, int k, in
                 if (a < m) v0 = __ldg(A + (size_t)r * m + a);
                 if (a + 1 < m) v1 = __ldg(A + (size_t)r * m + a + 1);
             }
-            float d0[kSlices], d1[kSlices];
-            oz_cut(v0, rs[u], d0);
-            oz_cut(v1, rs[u], d1);
+            uint32_t d[kSlices];
+            oz_cut(v0, v1, rs[u], rs[u], d);
 #pragma unroll
-            for (int s = 0; s < kSlices; ++s) sA[s * kGzPlane + rl * kGzStride + jl] = pack_bf16x2(d0[s], d1[s]);
+            for (int s = 0; s < kSlices; ++s) sA[s * kGzPlane + rl * kGzStride + jl] = d[s];
         }
         // V slices of this chunk: 32 columns x 16 k-pairs per slice
         for (int t = tid; t < kSlices * 32 * 16; t += kOzThreads) {
@@ -502,6 +549,145 @@ __global__ void __launch_bounds__(kOzThreads, 3) gemm_oz(int n, int m, int k, in
         }
 }
 
+// The same product with a CTA (8 warps of 16 x 8) per 32 rows of A and all
+// columns of C, for contractions up to kGrMaxK: the rows are read once, their
+// exponents found and their slices kept in shared memory, so a value is cut
+// once instead of once per 32 columns of C and no pass over A finds the
+// exponents; the slices of V stream through two stages of 32 columns x 32 steps
+// (cp.async).  n = 262,144, m = k = 150: 2.9 ms with 32 x 32 tiles, eight 7-bit
+// slices and an FP64 epilogue, 1.35 ms with this form (64-row CTAs, one per SM:
+// 1.43); the tensor pipe needs 0.63 at the rate of these instructions.
+static constexpr int kGrRows = 32, kGrThreads = 256, kGrMaxK = 320;
+
+static size_t gemm_rows_smem(int mp)
+{
+    return (size_t)kSlices * kGrRows * (mp / 2 + 4) * sizeof(uint32_t) + 2 * (size_t)kSlices * kGzPlane * sizeof(uint32_t) +
+           kGrRows * sizeof(int);
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t* dst, const uint32_t* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// Four 8 x 8 BF16 matrices from shared memory, rows of 16 bytes (lane l gives
+// the address of row l & 7 of matrix l >> 3).
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const uint32_t* p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+
+__global__ void __launch_bounds__(kGrThreads, 2) gemm_oz_rows(int n, int m, int k, int kp, int mp,
+                                                               const double* __restrict__ A, const uint32_t* __restrict__ Vs,
+                                                               const int* __restrict__ exV, double* __restrict__ C)
+{
+    extern __shared__ __align__(16) uint32_t gsm[];
+    const int half = mp / 2, ast = half + 4, aplane = kGrRows * ast;  // 4 words of padding: conflict-free fragments
+    uint32_t* sA = gsm;
+    uint32_t* sV = gsm + kSlices * aplane;  // two stages
+    int* sE = (int*)(sV + 2 * kSlices * kGzPlane);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int i0 = blockIdx.x * kGrRows;
+    const int nchunk = mp / 32, total = kp / 32 * nchunk;
+    auto stage = [&](int t) {  // slices of columns c0 .. c0 + 31, steps a0 .. a0 + 31
+        const int c0 = t / nchunk * 32, j0 = t % nchunk * 16;
+        uint32_t* dst = sV + (t & 1) * kSlices * kGzPlane;
+        for (int q = tid; q < kSlices * 32 * 4; q += kGrThreads) {
+            const int s = q / 128, cl = q / 4 % 32, v = q % 4;
+            cp_async16(dst + s * kGzPlane + cl * kGzStride + v * 4, Vs + ((size_t)s * kp + c0 + cl) * half + j0 + v * 4);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(0);
+    // rows of A: exponents and slices, a warp per row
+    for (int rl = warp; rl < kGrRows; rl += kGrThreads / 32) {
+        const int r = i0 + rl;
+        double v[kGrMaxK / 64][2];
+        int e = 0;
+#pragma unroll
+        for (int q = 0; q < kGrMaxK / 64; ++q)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = 2 * (lane + 32 * q) + h;
+                v[q][h] = r < n && c < m ? __ldg(A + (size_t)r * m + c) : 0.0;
+                e = max(e, (int)(((unsigned long long)__double_as_longlong(v[q][h]) >> 52) & 0x7ff));
+            }
+        for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+        const int E = oz_scale_exp(e);
+        if (lane == 0) sE[rl] = E;
+#pragma unroll
+        for (int q = 0; q < kGrMaxK / 64; ++q) {
+            const int j = lane + 32 * q;
+            if (j < half) {
+                uint32_t d[kSlices];
+                oz_cut(v[q][0], v[q][1], E, E, d);
+#pragma unroll
+                for (int s = 0; s < kSlices; ++s) sA[s * aplane + rl * ast + j] = d[s];
+            }
+        }
+    }
+    const int wr = (warp >> 2) * 16, wc = (warp & 3) * 8;
+    const int g = lane >> 2, tq = lane & 3;
+    // fragment addresses: A rows wr + (lane & 15), k half lane >> 4; V columns
+    // wc + (lane & 7), k quarter lane >> 3 (both halves of the chunk at once)
+    const uint32_t* fa = sA + (wr + (lane & 15)) * ast + (lane >> 4) * 4;
+    const int fv = (wc + (lane & 7)) * kGzStride + (lane >> 3) * 4;
+    float acc[kSlices][4];
+    long long ahi[4], alo[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        ahi[q] = alo[q] = 0;
+#pragma unroll
+        for (int l = 0; l < kSlices; ++l) acc[l][q] = 0.f;
+    }
+    for (int t = 0; t < total; ++t) {
+        const int chunk = t % nchunk;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();  // this stage is here, and everyone is done with the other
+        if (t + 1 < total) stage(t + 1);
+        const uint32_t* sv = sV + (t & 1) * kSlices * kGzPlane + fv;
+        uint32_t bf[kSlices][4];  // k quarters 0..3 of the chunk
+#pragma unroll
+        for (int s = 0; s < kSlices; ++s) ldsm4(bf[s], sv + s * kGzPlane);
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+            for (int s = 0; s < kSlices; ++s) {
+                uint32_t af[4];
+                ldsm4(af, fa + s * aplane + chunk * 16 + kk * 8);
+#pragma unroll
+                for (int t2 = 0; t2 < kSlices - s; ++t2)
+                    mma_bf16(acc[s + t2], af[0], af[1], af[2], af[3], bf[t2][2 * kk], bf[t2][2 * kk + 1]);
+            }
+        const bool end = chunk + 1 == nchunk;
+        if (end || chunk % kOzFlushChunks == kOzFlushChunks - 1) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float P[kSlices];
+#pragma unroll
+                for (int l = 0; l < kSlices; ++l) {
+                    P[l] = acc[l][q];
+                    acc[l][q] = 0.f;
+                }
+                oz_fold(P, ahi[q], alo[q]);
+            }
+        }
+        if (end) {
+            const int c0 = t / nchunk * 32;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int rl = wr + g + (q >= 2 ? 8 : 0), row = i0 + rl;
+                const int col = c0 + wc + 2 * tq + (q & 1);
+                if (row < n && col < k)
+                    C[(size_t)row * k + col] = oz_value(ahi[q], alo[q], sE[rl] + oz_scale_exp(__ldg(exV + col)));
+                ahi[q] = alo[q] = 0;
+            }
+        }
+    }
+}
+
 size_t gemm_oz_work_bytes(int n, int m, int k)
 {
     const size_t kp = (size_t)(k + 31) / 32 * 32, mp = (size_t)(m + 31) / 32 * 32;
@@ -520,11 +706,20 @@ cudaError_t launch_gemm_oz(int n, int m, int k, const double* A, const double* V
     uint32_t* Vs = (uint32_t*)p;
     cudaError_t e = cudaMemsetAsync(exV, 0, sizeof(int) * (size_t)k, s);
     if (e != cudaSuccess) return e;
-    int blocks = (int)std::min<long long>(((long long)n + 7) / 8, (long long)num_sms() * 8);
-    oz_rowexp<<<blocks, 256, 0, s>>>(n, m, A, exA);
     oz_colexp<<<std::max(1, std::min(m, 64)), 256, 0, s>>>(m, k, V, exV);
     const long long sv = (long long)kp * (mp / 2);
     oz_split_cols<<<(int)std::min<long long>((sv + 255) / 256, 1024), 256, 0, s>>>(m, k, kp, mp, V, exV, Vs);
+    if (mp <= kGrMaxK) {
+        const size_t smem = gemm_rows_smem(mp);
+        e = cudaFuncSetAttribute(gemm_oz_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_rows_smem(kGrMaxK));
+        if (e != cudaSuccess) return e;
+        gemm_oz_rows<<<(n + kGrRows - 1) / kGrRows, kGrThreads, smem, s>>>(n, m, k, kp, mp, A, Vs, exV, C);
+        count_launches(3);
+        return cudaGetLastError();
+    }
+    // longer contractions: their slices do not fit in shared memory
+    const int blocks = (int)std::min<long long>(((long long)n + 7) / 8, (long long)num_sms() * 8);
+    oz_rowexp<<<blocks, 256, 0, s>>>(n, m, A, exA);
     dim3 grid((n + 31) / 32, kp / 32);
     gemm_oz<<<grid, kOzThreads, 0, s>>>(n, m, k, kp, mp, A, Vs, exA, exV, C);
     count_launches(4);
