@@ -382,9 +382,7 @@ struct Bufs {
 
 size_t cplx_bytes(const Plan& P) { return P.fp64 ? 16 : 8; }
 
-// Device memory a contour pass may take for its Krylov bases, of one problem and
-// of a batch (which allocates per call).
-constexpr double kKrylovBytes = 64e9;
+// The same (kKrylovBytes) for a batch, which allocates its memory per call.
 constexpr double kKrylovBatchBytes = 8e9;
 
 Plan make_plan(int n, int nnzA, int nnzB, int m0, const int* fpm, bool filter_only = false)

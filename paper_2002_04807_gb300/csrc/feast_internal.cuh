@@ -177,6 +177,7 @@ struct KrylovArgs {
     int nunits, nteams, nc;
     int ne, nl, maxit, nbp, nbatch;
     int rii;
+    int cplx;           // rows are the real and imaginary parts of complex rows (R, X, Q complex blocks)
     int one_chunk;      // rows of at most eight entries, packed by krylov_pack (entries of row i at 8 i)
     double tol2;
     size_t slot_vecs, team_bytes;
@@ -196,8 +197,11 @@ struct KrylovArgs {
     const double* X;
     double* Q;
     int* iter_max;      // [problem][nbatch]
+    int* capped;        // pairs stopped by the step cap are added here, or nullptr
     unsigned long long* work;
 };
+// Device memory a contour pass of one problem may take for its Krylov bases.
+constexpr double kKrylovBytes = 64e9;
 KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes);
 KrylovPlan krylov_plan_set(bool fp64, int np, const int* n, const int* m, int ne, int maxit, double max_bytes);
 int krylov_rows(int n, int nc);  // rows per CTA of the resident form
@@ -205,6 +209,8 @@ size_t krylov_layout(const KrylovPlan& k, char* base, KrylovArgs& a);
 cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, cudaStream_t s);
 cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, bool fp64, void* out,
                                cudaStream_t s);
+cudaError_t launch_krylov_pack_hermitian(int n, const int* ia, const int* ja, const double2* av, const int* pp, bool fp64,
+                                         void* out, cudaStream_t s);
 cudaError_t launch_krylov_filter(const KrylovArgs& a, const KrylovPlan& p, bool fp64, cudaStream_t s);
 
 // persistent grid size of the COCG kernels: SMs x resident CTAs per SM

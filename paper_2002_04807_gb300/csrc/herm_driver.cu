@@ -128,6 +128,12 @@ struct HBufs {
     int ks;    // Gram split
     bool fp64;
     int* nactive_host;  // host copy of the two lane counters
+    KrylovPlan lz;      // B = I: one Krylov space per column (teams > 0), as the real path
+    KrylovArgs lza;
+    FiltProb* lzprob;   // its problem: 2 n real rows
+    int* lzpp;          // packed rows of the real operator
+    void* lzpk;
+    int* lzit;          // steps per node batch
     void* ozw;          // workspace of the sliced products (nullptr: FP64 DMMA products)
 };
 
@@ -138,9 +144,52 @@ struct HBufs {
 // read back every kCheckSteps steps; lanes that stop in between idle.
 constexpr int kCheckSteps = 8;
 
+// The pass from one Krylov space per column (k_krylov.cu): G(z_e) R and
+// G(conj z_e) R have conjugate coefficients in it, so the sum over both halves
+// of the contour is the real combination g = sum_e Re(c_e u_e) of the basis.
+// Four launches per BiCG step and node became one per pass (24^3, 60 columns:
+// the passes of a solve 130 -> 11 ms).
+int h_krylov_pass(HBufs& B, int ne, int rii, const double2* b, const double2* X, double tol, long long* iters,
+                  long long* capped, cudaStream_t s)
+{
+    KrylovArgs a = B.lza;
+    const int nbatch = (ne + B.nb - 1) / B.nb;
+    a.probs = B.lzprob;
+    a.nunits = (B.fa.m + B.lz.cols - 1) / B.lz.cols;
+    a.nbp = B.nb;
+    a.nbatch = nbatch;
+    a.rii = rii;
+    a.cplx = 1;
+    a.tol2 = tol * tol;
+    a.err = B.nactive;
+    a.limit = wait_limit_cycles();
+    a.R = (const double*)b;
+    a.X = (const double*)X;
+    a.Q = (double*)B.Q;
+    a.iter_max = B.lzit;
+    a.capped = B.nactive + 1;
+    HCK(cudaMemsetAsync(B.lzit, 0, sizeof(int) * nbatch, s));
+    HCK(cudaMemsetAsync(B.nactive, 0, 2 * sizeof(int), s));
+    HCK(cudaMemsetAsync(a.bar, 0, sizeof(unsigned) * ((size_t)a.nteams * 32 + 32), s));
+    HCK(launch_krylov_filter(a, B.lz, B.fp64, s));
+    std::vector<int> it(nbatch);
+    int h[2] = {0, 0};
+    HCK(cudaMemcpyAsync(it.data(), B.lzit, sizeof(int) * nbatch, cudaMemcpyDeviceToHost, s));
+    HCK(cudaMemcpyAsync(h, B.nactive, sizeof(h), cudaMemcpyDeviceToHost, s));
+    HCK(cudaStreamSynchronize(s));
+    if (h[0]) return cuda_error(cudaErrorLaunchTimeout, "contour filter: a wait exceeded the wait limit");
+    for (const int k : it) *iters += k;
+    *capped += h[1];
+    return 0;
+}
+
 int h_filter_pass(HBufs& B, const HMat& A, const HMat& Bm, bool hasB, int m, int ne, int rii, const double2* b,
                   const double2* X, int maxit, double tol, long long* iters, long long* capped, cudaStream_t s)
 {
+    if (B.lz.teams > 0) {
+        B.fa.m = m;
+        return h_krylov_pass(B, ne, rii, b, X, tol, iters, capped, s);
+    }
     HArgs a = B.fa;
     a.n = A.n;
     a.m = m;
@@ -186,6 +235,7 @@ struct HPlan {
     long long Lmax = 0;
     bool fp64 = false, hasB = false;
     bool oz = true;  // fpm(54) = 0: projections and Ritz vectors from sliced BF16 products
+    KrylovPlan lz;   // B = I and the basis fits: one Krylov space per column
 };
 
 HPlan h_plan(int n, int nnz_a, int nnz_b, int m0, const int* fpm)
@@ -204,6 +254,9 @@ HPlan h_plan(int n, int nnz_a, int nnz_b, int m0, const int* fpm)
     P.Lmax = (long long)m0 * P.nbp;
     h_gram_partial(n, m0, &P.ks);
     P.oz = fpm[53] == 0;
+    // (rows and packed entries of the real operator counted in 32-bit ints)
+    if (!P.hasB && n <= (1 << 30) && 4.0 * nnz_a + 14.0 * n < 2147483647.0)
+        P.lz = krylov_plan(P.fp64, false, 2 * n, m0, P.ne, fpm[45], kKrylovBytes);
     return P;
 }
 
@@ -245,12 +298,23 @@ size_t h_carve(const HPlan& P, void* base, HBufs& B, float2** af, float2** bf)
     B.nactive = c.take<int>(2);
     B.perm = c.take<int>(P.m0);
     B.red = c.take<char>(h_reduced_work_bytes(P.m0));
+    B.lz = P.lz;
+    const bool lz = P.lz.teams > 0;
+    if (lz) {
+        KrylovArgs t = {};
+        char* mem = c.take<char>(krylov_layout(P.lz, nullptr, t));
+        if (base) krylov_layout(P.lz, mem, B.lza);
+        B.lzprob = c.take<FiltProb>(1);
+        B.lzpp = c.take<int>(2 * (size_t)P.n + 1);
+        B.lzpk = c.take<char>((4 * (size_t)P.nnz_a + 14 * (size_t)P.n) * (P.fp64 ? 16 : 8));
+        B.lzit = c.take<int>(P.ne);
+    }
     void** fv[6] = {&B.fa.r, &B.fa.rh, &B.fa.p, &B.fa.ph, &B.fa.q, &B.fa.qh};
-    for (void** v : fv) *v = c.take<char>((size_t)P.n * P.Lmax * vb);
-    B.fa.dQ = P.fp64 ? nullptr : c.take<float2>(blk);
-    B.fa.st = c.take<HLane>(P.Lmax);
-    B.fa.part = c.take<double2>((size_t)row_blocks(P.n) * 2 * P.Lmax);
-    *af = P.fp64 ? nullptr : c.take<float2>(P.nnz_a);
+    for (void** v : fv) *v = c.take<char>(lz ? 0 : (size_t)P.n * P.Lmax * vb);
+    B.fa.dQ = P.fp64 || lz ? nullptr : c.take<float2>(blk);
+    B.fa.st = c.take<HLane>(lz ? 0 : P.Lmax);
+    B.fa.part = c.take<double2>(lz ? 0 : (size_t)row_blocks(P.n) * 2 * P.Lmax);
+    *af = P.fp64 || lz ? nullptr : c.take<float2>(P.nnz_a);
     *bf = (P.fp64 || !P.hasB) ? nullptr : c.take<float2>(P.nnz_b);
     B.ozw = P.oz ? c.take<char>(h_sliced_work_bytes(P.n, P.m0)) : nullptr;
     return c.off + 256;
@@ -448,7 +512,27 @@ static int h_dev_entry(int n, int nnz_a, const int* d_ia, const int* d_ja, const
         Bm.v = (const double2*)d_b;
         Bm.vf = d_b;
     }
-    if (!P.fp64) {  // complex float copies of the values for the filter
+    if (P.lz.teams > 0) {  // the matrix as a real operator on real and imaginary parts
+        std::vector<int> ia(n + 1), pp(2 * (size_t)n + 1, 0);
+        cudaError_t ce = cudaMemcpyAsync(ia.data(), d_ia, sizeof(int) * (n + 1), cudaMemcpyDeviceToHost, s);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+        for (int i = 0; i < 2 * n; ++i) pp[i + 1] = pp[i] + (2 * (ia[i / 2 + 1] - ia[i / 2]) + 7) / 8 * 8;
+        FiltProb fp;
+        memset(&fp, 0, sizeof(fp));
+        fp.n = 2 * n;
+        fp.m0 = *m0;
+        fp.app = B.lzpp;
+        fp.apk = B.lzpk;
+        fp.zw = B.zw;
+        fp.lam = B.lam;
+        fp.ne = P.ne;
+        fp.active = 1;
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(B.lzpp, pp.data(), sizeof(int) * pp.size(), cudaMemcpyHostToDevice, s);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(B.lzprob, &fp, sizeof(fp), cudaMemcpyHostToDevice, s);
+        if (ce == cudaSuccess) ce = launch_krylov_pack_hermitian(n, d_ia, d_ja, A.v, B.lzpp, P.fp64, B.lzpk, s);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);  // pp and fp are host temporaries
+        if (ce != cudaSuccess) return ret(cuda_error(ce, "packed rows"));
+    } else if (!P.fp64) {  // complex float copies of the values for the filter
         cudaError_t ce = launch_h_cast(A.v, af, nnz_a, false, s);
         if (ce != cudaSuccess) return ret(cuda_error(ce, "cast"));
         A.vf = af;

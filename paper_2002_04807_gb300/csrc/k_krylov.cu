@@ -324,6 +324,11 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
         const int4* __restrict__ ent = (const int4*)P.apk;
         const int* __restrict__ app = P.app;
         const int col0 = g * COLS + l * N;  // the thread's first column
+        // element of the FP64 blocks: row-major, or the real (even row) or imaginary
+        // part (odd row) of a complex block
+        auto elem = [&](int i, int col) {
+            return P.q_off + (a.cplx ? ((size_t)(i >> 1) * m0 + col) * 2 + (i & 1) : (size_t)i * m0 + col);
+        };
         auto row_of = [&](int t) { return lz_row<RES, PASS>(t, slot, r0, c, nc); };
 
         // ---- init: u_1 = b
@@ -334,7 +339,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
             LzPack<T> x;
 #pragma unroll
             for (int q = 0; q < N; ++q) {
-                x.e[q] = col0 + q < mk ? (T)a.R[P.q_off + (size_t)i * m0 + col0 + q] : T(0);
+                x.e[q] = col0 + q < mk ? (T)a.R[elem(i, col0 + q)] : T(0);
                 acc[q].add(x.e[q] * x.e[q]);
             }
             basis[(size_t)i * LPR + l] = x.v;
@@ -642,7 +647,10 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
         if (c == 0) {
             for (int pr = tid; pr < npair; pr += kLzThreads) {
                 int ks = kst[pr];
-                if (ks < 0) kst[pr] = ks = k;
+                if (ks < 0) {
+                    kst[pr] = ks = k;
+                    if (a.capped) atomicAdd(a.capped, 1);
+                }
                 atomicMax(a.iter_max + (size_t)un.x * a.nbatch + (pr / COLS) / a.nbp, max(ks, 1));
             }
             if (tid == 0 && a.work) atomicAdd(a.work, (unsigned long long)k);
@@ -743,7 +751,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
 #pragma unroll
             for (int q = 0; q < N; ++q)
                 if (col0 + q < m0) {
-                    const size_t o = P.q_off + (size_t)i * m0 + col0 + q;
+                    const size_t o = elem(i, col0 + q);
                     double v = 0.0;
                     if (col0 + q < mk) v = (a.rii ? rq[q] * a.X[o] : 0.0) + (double)sum.e[q];
                     a.Q[o] = v;
@@ -852,6 +860,48 @@ cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, con
     const int grid = std::max(1, std::min((n + 31) / 32, num_sms() * 16));
     if (fp64) krylov_pack<int4><<<grid, 256, 0, s>>>(n, rpc, ia, ja, av, (int4*)out);
     else krylov_pack<int2><<<grid, 256, 0, s>>>(n, rpc, ia, ja, av, (int2*)out);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------- complex Hermitian matrices
+// Lanczos on a Hermitian A has real coefficients, so it is real Lanczos on the
+// real symmetric operator that takes (Re x, Im x) to (Re A x, Im A x).  Rows 2 i
+// and 2 i + 1 of that operator hold row i's entries as (2 j, Re a), (2 j + 1,
+// -Im a) and (2 j, Im a), (2 j + 1, Re a), padded to chunks of eight at pp.
+template <typename E, typename V2>
+__global__ void __launch_bounds__(256) krylov_pack_hermitian(int n, const int* __restrict__ ia, const int* __restrict__ ja,
+                                                             const V2* __restrict__ av, const int* __restrict__ pp,
+                                                             E* __restrict__ out)
+{
+    const int lane = threadIdx.x & 31, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
+        const int p0 = ia[i], len = ia[i + 1] - p0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c0 = pp[2 * i + h], c1 = pp[2 * i + h + 1];
+            for (int t = c0 + lane; t < c1; t += 32) {
+                const int q = (t - c0) >> 1, im = (t - c0) & 1;
+                int j = -1;
+                double v = 0.0;
+                if (q < len) {
+                    j = 2 * ja[p0 + q] + im;
+                    const V2 a = av[p0 + q];
+                    v = im == h ? (double)a.x : (h ? (double)a.y : -(double)a.y);
+                }
+                if constexpr (sizeof(E) == 8) out[t] = make_int2(j, __float_as_int((float)v));
+                else out[t] = make_int4(j, 0, __double2loint(v), __double2hiint(v));
+            }
+        }
+    }
+}
+
+cudaError_t launch_krylov_pack_hermitian(int n, const int* ia, const int* ja, const double2* av, const int* pp, bool fp64,
+                                         void* out, cudaStream_t s)
+{
+    const int grid = std::max(1, std::min((n + 7) / 8, num_sms() * 16));
+    if (fp64) krylov_pack_hermitian<int4><<<grid, 256, 0, s>>>(n, ia, ja, av, pp, (int4*)out);
+    else krylov_pack_hermitian<int2><<<grid, 256, 0, s>>>(n, ia, ja, av, pp, (int2*)out);
     count_launches(1);
     return cudaGetLastError();
 }
