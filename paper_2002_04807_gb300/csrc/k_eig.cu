@@ -142,21 +142,21 @@ __global__ void __launch_bounds__(kEigThreads) jacobi_team(JacArgs a)
         int* rp = (int*)(rt + half);
         int* rq = rp + half;
         for (long long idx = gtid; idx < (long long)m * m; idx += gsz) V[idx] = (idx / m == idx % m) ? 1.0 : 0.0;
-        double fr = 0.0;  // every CTA sums the same entries in the same order
-        for (long long idx = threadIdx.x; idx < (long long)m * m; idx += blockDim.x)
-            fr += fabs(A[idx]) < 1e299 ? A[idx] * A[idx] : 0.0;  // sentinels excluded
+        double fr = 0.0;  // the largest entry, the same in every CTA
+        for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x)
+            if (fabs(A[idx]) < 1e299) fr = fmax(fr, fabs(A[idx]));  // sentinels excluded
         sred[threadIdx.x] = fr;
         __syncthreads();
         for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) sred[threadIdx.x] += sred[threadIdx.x + o];
+            if (threadIdx.x < o) sred[threadIdx.x] = fmax(sred[threadIdx.x], sred[threadIdx.x + o]);
             __syncthreads();
         }
-        const double fro = sqrt(sred[0]);
+        const double big = sred[0];
         if (cta == 0 && threadIdx.x == 0) w->again[0] = w->again[1] = 0;
         if (!team_sync(&w->count, target, nc, &w->err, a.limit)) return;
-        const double sc = fro > 0.0 && fro < 1e300 ? ldexp(1.0, -ilogb(fro)) : 1.0;
+        const double sc = big > 1e-300 && big < 1e300 ? ldexp(1.0, -ilogb(big)) : 1.0;
         // |x| above 1.1e-16 sqrt(|xp xq|) and the floor of 1e-18 of the matrix, all
-        // scaled by sc: the norm is near 1, nothing under- or overflows
+        // scaled by sc: the largest entry is near 1, nothing under- or overflows
         auto above = [](float x, float xp, float xq) {
             return fabsf(x) > 1e-18f && x * x > 1.21e-32f * fabsf(xp) * fabsf(xq);
         };

@@ -33,6 +33,7 @@
 
 #include "feast_internal.cuh"
 #include "herm_internal.cuh"
+#include "team.cuh"
 
 namespace feast {
 namespace herm {
@@ -1126,52 +1127,36 @@ cudaError_t launch_h_jacobi(int m, double2* A, double2* Vw, double* lam, double2
 }
 
 // ---------------------------------------------------------------- Hermitian Jacobi (many CTAs)
-// The same rotations as h_jacobi, spread over the CTAs of one cooperative
-// launch with one grid barrier per round (GB300's FP64 rate per SM is low, so
-// one CTA is slow): every CTA computes all rotations of the round (identical
-// inputs and code, so identical angles) into shared memory, then updates its
-// share of the 2 x 2 blocks from the current copy of A into the other copy,
-// so no CTA writes what another still reads.  Block (k, l) holds rows p_k, q_k
-// and columns p_l, q_l; with J_k = D_k R_k (columns (c, -s conj e) and
-// (s, c conj e)) it becomes J_k^H A J_l; a diagonal block becomes
-// diag(a_pp - t |a_pq|, a_qq + t |a_pq|).  The barrier spins at most
-// wait_limit_cycles() cycles, then every CTA returns and *err is set.
+// The rotations of h_jacobi spread over the CTAs of one cooperative launch, one
+// barrier per round, as jacobi_team does for real matrices (k_eig.cu): every
+// CTA computes all rotations of the round (identical inputs and code, so
+// identical angles) into shared memory, then its share of the 2 x 2 blocks from
+// the current copy of A into the other copy, so no CTA writes what another
+// still reads; of two blocks that are each other's conjugate transpose one is
+// computed and written twice.  Block (k, l) holds rows p_k, q_k and columns
+// p_l, q_l; with J_k = D_k R_k (columns (c, -s conj e) and (s, c conj e)) it
+// becomes J_k^H A J_l.  With e = a_pq / |a_pq| the diagonal block is that of the
+// real rotation of (a_pp, |a_pq|, a_qq); t comes from a single-precision root
+// and one Newton step, and -c^2 f(t), about 1e-13 of a_pq, is what is left in
+// the place of a_pq.  hypot, four divisions and two square roots per angle in
+// every CTA, and a last sweep that found nothing, took 3.7 ms at m = 60, now
+// 2.3.  The barrier gives up after the wait limit: every CTA returns and
+// err is set.
 struct HJWork {
-    unsigned long long count;  // barrier arrivals since launch; never reset
+    unsigned count;  // barrier arrivals
     int err;
     int sweeps;
     int status;
-    int pad;
-    double fro;
+    int again[2];  // a sweep left an entry above the threshold
 };
 
-__device__ __forceinline__ bool h_grid_sync(HJWork* w, long long limit)
+// 1 / sqrt(y) for y within single-precision range: a seed and two Newton steps.
+__device__ __forceinline__ double h_rsqrt(double y)
 {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int good = (*(volatile int*)&w->err == 0);
-        if (good) {
-            unsigned long long old;
-            asm volatile("atom.add.release.gpu.u64 %0, [%1], 1;" : "=l"(old) : "l"(&w->count) : "memory");
-            const unsigned long long target = (old / gridDim.x + 1) * gridDim.x;
-            const long long t0 = clock64();
-            for (;;) {
-                unsigned long long cur;
-                asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(cur) : "l"(&w->count) : "memory");
-                if (cur >= target) break;
-                if (*(volatile int*)&w->err) { good = 0; break; }
-                if (clock64() - t0 > limit) {
-                    atomicExch(&w->err, 1);
-                    good = 0;
-                    break;
-                }
-            }
-        }
-        ok = good;
-    }
-    __syncthreads();
-    return ok != 0;
+    double r = (double)rsqrtf((float)y);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) r = r * fma(-0.5 * y * r, r, 1.5);
+    return r;
 }
 
 __global__ void __launch_bounds__(256) h_jacobi_coop(int m, double2* __restrict__ A, double2* __restrict__ A2,
@@ -1182,61 +1167,99 @@ __global__ void __launch_bounds__(256) h_jacobi_coop(int m, double2* __restrict_
     __shared__ double s_c[kHJMax / 2], s_s[kHJMax / 2], s_t[kHJMax / 2];
     __shared__ double2 s_e[kHJMax / 2];
     __shared__ int s_p[kHJMax / 2], s_q[kHJMax / 2];
-    __shared__ double s_red[8];
-    __shared__ int s_any;
-    const int N = (m + 1) & ~1, half = N / 2;
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
-    for (long long idx = gtid; idx < (long long)m * m; idx += gsz)
-        Vw[idx] = make_double2(idx / m == idx % m ? 1.0 : 0.0, 0.0);
-    if (blockIdx.x == 0) {  // Frobenius norm, fixed order
-        double f = 0.0;
-        for (long long idx = threadIdx.x; idx < (long long)m * m; idx += blockDim.x) {
-            const double2 v = A[idx];
-            f = fma(v.x, v.x, fma(v.y, v.y, f));
-        }
-        for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-        if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = f;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += s_red[i];
-            w->fro = sqrt(t);
-        }
+    __shared__ double s_red[256];
+    const int N = (m + 1) & ~1, half = N / 2, nc = gridDim.x;
+    const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsz = nc * blockDim.x;
+    unsigned target = 0;
+    for (int idx = gtid; idx < m * m; idx += gsz) Vw[idx] = make_double2(idx / m == idx % m ? 1.0 : 0.0, 0.0);
+    double f = 0.0;  // the largest entry, the same in every CTA
+    for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
+        const double2 v = A[idx];
+        f = fmax(f, fmax(fabs(v.x), fabs(v.y)));
     }
-    if (!h_grid_sync(w, limit)) return;
-    const double absfloor = 1e-18 * *(volatile double*)&w->fro;
+    s_red[threadIdx.x] = f;
+    __syncthreads();
+    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) s_red[threadIdx.x] = fmax(s_red[threadIdx.x], s_red[threadIdx.x + o]);
+        __syncthreads();
+    }
+    const double big = s_red[0];
+    if (!team_sync(&w->count, target, nc, &w->err, limit)) return;
+    const double sc = big > 1e-300 && big < 1e300 ? ldexp(1.0, -ilogb(big)) : 1.0;
+    // squared size x2 above that of 1.1e-16 sqrt(|xp xq|) and of the floor, all scaled by sc
+    auto above = [](float x2, float xp, float xq) { return x2 > 1e-36f && x2 > 1.21e-32f * fabsf(xp) * fabsf(xq); };
+    auto pair = [&](int k, int r, int& p, int& q) {  // round-robin: (r, N-1), (r + k, r - k) mod N - 1
+        p = r + k;
+        if (p >= N - 1) p -= N - 1;
+        q = k ? r - k : N - 1;
+        if (q < 0) q += N - 1;
+        if (p > q) {
+            const int t = p;
+            p = q;
+            q = t;
+        }
+    };
+    // every unordered pair of pairs {k, l} once; the diagonal blocks after the others
+    const int ncol = half / 2, nblk = half * (ncol + 1);
+    auto block = [&](int idx, int& k, int& l) {
+        if (idx >= half * ncol) {
+            k = l = idx - half * ncol;
+            return idx < nblk;
+        }
+        k = idx / ncol;
+        const int d = idx - k * ncol + 1;
+        l = k + d < half ? k + d : k + d - half;
+        return 2 * d < half || k < half / 2;
+    };
     double2* cur = A;
     double2* nxt = A2;
+    const double2 z0 = make_double2(0.0, 0.0);
+    int k0 = 0, l0 = 0;
+    const bool has = block(gtid, k0, l0), hasv = gtid < m * half;
+    const int i0 = gtid / half, kv0 = gtid - i0 * half;
     int sweep = 0;
     bool more = m > 1;
     while (more && sweep < kHJSweeps) {
-        if (threadIdx.x == 0) s_any = 0;
-        __syncthreads();
         for (int r = 0; r < N - 1; ++r) {
+            double2 x00 = z0, x01 = z0, x10 = z0, x11 = z0, vp = z0, vq = z0;
+            auto load = [&](int p, int q, int pp, int qq) {
+                x00 = __ldcg(cur + (size_t)p * m + pp);
+                x01 = qq < m ? __ldcg(cur + (size_t)p * m + qq) : z0;
+                x10 = q < m ? __ldcg(cur + (size_t)q * m + pp) : z0;
+                x11 = q < m && qq < m ? __ldcg(cur + (size_t)q * m + qq) : z0;
+            };
+            if (has) {
+                int p, q, pp, qq;
+                pair(k0, r, p, q);
+                pair(l0, r, pp, qq);
+                load(p, q, pp, qq);
+            }
+            if (hasv) {
+                int p, q;
+                pair(kv0, r, p, q);
+                vp = __ldcg(Vw + (size_t)i0 * m + p);
+                vq = q < m ? __ldcg(Vw + (size_t)i0 * m + q) : z0;
+            }
             for (int k = threadIdx.x; k < half; k += blockDim.x) {
                 int p, q;
-                if (k == 0) {
-                    p = r;
-                    q = N - 1;
-                } else {
-                    p = (r + k) % (N - 1);
-                    q = (r - k + (N - 1)) % (N - 1);
-                }
-                if (p > q) { const int t = p; p = q; q = t; }
+                pair(k, r, p, q);
                 double c = 1.0, s = 0.0, tt = 0.0;
                 double2 e = make_double2(1.0, 0.0);
                 if (q < m) {
                     const double2 apq = __ldcg(cur + (size_t)p * m + q);
-                    const double mag = hypot(apq.x, apq.y);
-                    const double app = __ldcg(cur + (size_t)p * m + p).x, aqq = __ldcg(cur + (size_t)q * m + q).x;
-                    const double thr = fmax(1.1e-16 * sqrt(fabs(app * aqq)), absfloor);
-                    if (mag > thr) {
-                        e = make_double2(apq.x / mag, apq.y / mag);
-                        const double tau = (aqq - app) / (2.0 * mag);
-                        tt = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        c = 1.0 / sqrt(1.0 + tt * tt);
+                    const double bx = apq.x * sc, by = apq.y * sc;
+                    const double xp = __ldcg(cur + (size_t)p * m + p).x * sc, xq = __ldcg(cur + (size_t)q * m + q).x * sc;
+                    const double b2 = fma(bx, bx, by * by);
+                    if (above((float)b2, (float)xp, (float)xq)) {
+                        const double ri = h_rsqrt(b2);
+                        e = make_double2(bx * ri, by * ri);
+                        const double b = b2 * ri, d = xq - xp;
+                        const float df = (float)d, bf = (float)b, h = 0.5f * df;
+                        const float x = df == 0.0f ? 1.0f : copysignf(1.0f, h) * (bf / (fabsf(h) + sqrtf(fmaf(h, h, bf * bf))));
+                        tt = (double)x;
+                        tt = fma(-fma(fma(b, tt, d), tt, -b), (double)(1.0f / fmaf(2.0f * bf, x, df)), tt);
+                        c = h_rsqrt(fma(tt, tt, 1.0));
                         s = tt * c;
-                        s_any = 1;
                     }
                 }
                 s_c[k] = c;
@@ -1247,38 +1270,36 @@ __global__ void __launch_bounds__(256) h_jacobi_coop(int m, double2* __restrict_
                 s_q[k] = q;
             }
             __syncthreads();
-            for (long long idx = gtid; idx < (long long)half * half; idx += gsz) {
-                const int k = (int)(idx / half), l = (int)(idx % half);
+            for (int idx = gtid; idx < nblk; idx += gsz) {
+                int k = k0, l = l0;
+                if (idx == gtid ? !has : !block(idx, k, l)) continue;
                 const int p = s_p[k], q = s_q[k], pp = s_p[l], qq = s_q[l];
                 const bool qv = q < m, qqv = qq < m;
+                if (idx != gtid) load(p, q, pp, qq);
+                const double2 ek = s_e[k], el = s_e[l];
                 if (k == l) {
-                    const double2 app = __ldcg(cur + (size_t)p * m + p);
+                    const double t = s_t[k], app = x00.x, aqq = x11.x;
                     if (!qv) {
-                        nxt[(size_t)p * m + p] = make_double2(app.x, 0.0);
+                        nxt[(size_t)p * m + p] = make_double2(app, 0.0);
                         continue;
                     }
-                    const double2 apq = __ldcg(cur + (size_t)p * m + q), aqq = __ldcg(cur + (size_t)q * m + q);
                     if (s_s[k] == 0.0) {
-                        nxt[(size_t)p * m + p] = make_double2(app.x, 0.0);
-                        nxt[(size_t)q * m + q] = make_double2(aqq.x, 0.0);
-                        nxt[(size_t)p * m + q] = apq;
-                        nxt[(size_t)q * m + p] = __ldcg(cur + (size_t)q * m + p);
-                    } else {
-                        const double mag = hypot(apq.x, apq.y);
-                        nxt[(size_t)p * m + p] = make_double2(app.x - s_t[k] * mag, 0.0);
-                        nxt[(size_t)q * m + q] = make_double2(aqq.x + s_t[k] * mag, 0.0);
-                        nxt[(size_t)p * m + q] = make_double2(0.0, 0.0);
-                        nxt[(size_t)q * m + p] = make_double2(0.0, 0.0);
+                        nxt[(size_t)p * m + p] = make_double2(app, 0.0);
+                        nxt[(size_t)q * m + q] = make_double2(aqq, 0.0);
+                        nxt[(size_t)p * m + q] = x01;
+                        nxt[(size_t)q * m + p] = make_double2(x01.x, -x01.y);
+                        continue;
                     }
+                    // the real rotation of (app, |apq|, aqq), with f(t)
+                    const double mag = fma(ek.x, x01.x, ek.y * x01.y);
+                    const double g = s_c[k] * s_c[k] * fma(fma(mag, t, aqq - app), t, -mag);
+                    const double ta = fma(-t, g, t * mag);
+                    nxt[(size_t)p * m + p] = make_double2(app - ta, 0.0);
+                    nxt[(size_t)q * m + q] = make_double2(aqq + ta, 0.0);
+                    nxt[(size_t)p * m + q] = nxt[(size_t)q * m + p] = make_double2(-g, 0.0);
                     continue;
                 }
                 const double ck = s_c[k], sk = s_s[k], cl = s_c[l], sl = s_s[l];
-                const double2 ek = s_e[k], el = s_e[l];
-                const double2 z = make_double2(0.0, 0.0);
-                const double2 x00 = __ldcg(cur + (size_t)p * m + pp);
-                const double2 x01 = qqv ? __ldcg(cur + (size_t)p * m + qq) : z;
-                const double2 x10 = qv ? __ldcg(cur + (size_t)q * m + pp) : z;
-                const double2 x11 = (qv && qqv) ? __ldcg(cur + (size_t)q * m + qq) : z;
                 // rows (J_k^H): y0 = c x0 - s e x1, y1 = s x0 + c e x1
                 const double2 ex10 = make_double2(ek.x * x10.x - ek.y * x10.y, ek.x * x10.y + ek.y * x10.x);
                 const double2 ex11 = make_double2(ek.x * x11.x - ek.y * x11.y, ek.x * x11.y + ek.y * x11.x);
@@ -1290,41 +1311,74 @@ __global__ void __launch_bounds__(256) h_jacobi_coop(int m, double2* __restrict_
                 const double2 ec = make_double2(el.x, -el.y);
                 const double2 ey01 = make_double2(ec.x * y01.x - ec.y * y01.y, ec.x * y01.y + ec.y * y01.x);
                 const double2 ey11 = make_double2(ec.x * y11.x - ec.y * y11.y, ec.x * y11.y + ec.y * y11.x);
-                nxt[(size_t)p * m + pp] = make_double2(cl * y00.x - sl * ey01.x, cl * y00.y - sl * ey01.y);
-                if (qqv) nxt[(size_t)p * m + qq] = make_double2(sl * y00.x + cl * ey01.x, sl * y00.y + cl * ey01.y);
-                if (qv) nxt[(size_t)q * m + pp] = make_double2(cl * y10.x - sl * ey11.x, cl * y10.y - sl * ey11.y);
-                if (qv && qqv)
-                    nxt[(size_t)q * m + qq] = make_double2(sl * y10.x + cl * ey11.x, sl * y10.y + cl * ey11.y);
+                auto put = [&](int row, int col, double2 v) {
+                    nxt[(size_t)row * m + col] = v;
+                    nxt[(size_t)col * m + row] = make_double2(v.x, -v.y);
+                };
+                put(p, pp, make_double2(cl * y00.x - sl * ey01.x, cl * y00.y - sl * ey01.y));
+                if (qqv) put(p, qq, make_double2(sl * y00.x + cl * ey01.x, sl * y00.y + cl * ey01.y));
+                if (qv) put(q, pp, make_double2(cl * y10.x - sl * ey11.x, cl * y10.y - sl * ey11.y));
+                if (qv && qqv) put(q, qq, make_double2(sl * y10.x + cl * ey11.x, sl * y10.y + cl * ey11.y));
             }
-            for (long long idx = gtid; idx < (long long)m * half; idx += gsz) {  // V <- V J
-                const int i = (int)(idx / half), k = (int)(idx % half);
+            for (int idx = gtid; idx < m * half; idx += gsz) {  // V <- V J
+                const int i = idx == gtid ? i0 : idx / half, k = idx == gtid ? kv0 : idx - i * half;
                 const double sk = s_s[k];
                 if (sk == 0.0) continue;
                 const double ck = s_c[k];
                 const double2 ec = make_double2(s_e[k].x, -s_e[k].y);
                 const int p = s_p[k], q = s_q[k];
-                const double2 vp = Vw[(size_t)i * m + p], vq = Vw[(size_t)i * m + q];
+                if (idx != gtid) {
+                    vp = __ldcg(Vw + (size_t)i * m + p);
+                    vq = __ldcg(Vw + (size_t)i * m + q);
+                }
                 const double2 evq = make_double2(ec.x * vq.x - ec.y * vq.y, ec.x * vq.y + ec.y * vq.x);
                 Vw[(size_t)i * m + p] = make_double2(ck * vp.x - sk * evq.x, ck * vp.y - sk * evq.y);
                 Vw[(size_t)i * m + q] = make_double2(sk * vp.x + ck * evq.x, sk * vp.y + ck * evq.y);
             }
-            if (!h_grid_sync(w, limit)) return;
+            if (!team_sync(&w->count, target, nc, &w->err, limit)) return;
             double2* tmp = cur;
             cur = nxt;
             nxt = tmp;
         }
-        more = s_any != 0;  // same decision in every CTA
+        // entries still above the threshold?
+        int rest = 0;
+        for (int idx = gtid; idx < m * m; idx += gsz) {
+            const int i = idx / m, j = idx % m;
+            if (j <= i) continue;
+            const double2 x = __ldcg(cur + idx);
+            const double bx = x.x * sc, by = x.y * sc;
+            if (above((float)fma(bx, bx, by * by), (float)(__ldcg(cur + (size_t)i * m + i).x * sc),
+                      (float)(__ldcg(cur + (size_t)j * m + j).x * sc)))
+                rest = 1;
+        }
+        if (__syncthreads_or(rest) && threadIdx.x == 0) *(volatile int*)&w->again[sweep & 1] = 1;
+        if (!team_sync(&w->count, target, nc, &w->err, limit)) return;
+        more = *(volatile int*)&w->again[sweep & 1] != 0;  // same decision in every CTA
+        // the other flag is read next; nobody reads it before the next barrier
+        if (gtid == 0) *(volatile int*)&w->again[(sweep & 1) ^ 1] = 0;
         ++sweep;
     }
-    for (int i = gtid; i < m; i += gsz) {  // ascending order: rank by value, ties by index
-        const double li = __ldcg(cur + (size_t)i * m + i).x;
-        int rk = 0;
-        for (int j = 0; j < m; ++j) {
-            const double lj = __ldcg(cur + (size_t)j * m + j).x;
-            rk += (lj < li) || (lj == li && j < i);
+    // ascending order: rank by value, ties by index (the rotation tables are free)
+    double* dg = (double*)s_e;
+    int* rank = s_p;
+    for (int part = 0; part < m; part += kHJMax / 2) {  // ranks of half the table at a time
+        __syncthreads();
+        for (int i = threadIdx.x; i < m; i += blockDim.x) dg[i] = __ldcg(cur + (size_t)i * m + i).x;
+        __syncthreads();
+        const int end = min(m, part + kHJMax / 2);
+        for (int i = part + threadIdx.x; i < end; i += blockDim.x) {
+            const double li = dg[i];
+            int rk = 0;
+            for (int j = 0; j < m; ++j) rk += (dg[j] < li) || (dg[j] == li && j < i);
+            rank[i - part] = rk;
+            if (blockIdx.x == 0) lam[rk] = li;
         }
-        lam[rk] = li;
-        for (int row = 0; row < m; ++row) Vout[(size_t)row * m + rk] = Vw[(size_t)row * m + i];
+        __syncthreads();
+        const int wd = end - part;
+        for (int idx = gtid; idx < m * wd; idx += gsz) {
+            const int row = idx / wd, i = idx % wd;
+            Vout[(size_t)row * m + rank[i]] = __ldcg(Vw + (size_t)row * m + part + i);
+        }
     }
     if (gtid == 0) {
         w->sweeps = sweep;
@@ -1348,16 +1402,10 @@ static cudaError_t launch_h_jacobi_coop(int m, double2* A, double* lam, double2*
     double2* Vw = A2 + (size_t)m * m;
     cudaError_t e = cudaMemsetAsync(w, 0, sizeof(HJWork), s);
     if (e != cudaSuccess) return e;
-    static const int per_sm = [] {
-        int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, h_jacobi_coop, 256, 0);
-        return v > 0 ? v : 1;
-    }();
-    const int half = (m + 1) / 2;
-    long long blocks = ((long long)m * half + 255) / 256;
-    const long long cap = std::min<long long>((long long)num_sms() * per_sm, num_sms());
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
+    // a warp instruction holds the FP64 pipe for 16 cycles however few lanes work:
+    // a warp of blocks per CTA
+    const long long half = (m + 1) / 2;
+    const long long blocks = std::max(1LL, std::min<long long>((half * (half / 2 + 1) + 31) / 32, num_sms()));
     long long limit = wait_limit_cycles();
     void* args[] = {&m, &A, &A2, &Vw, &lam, &V, &w, &limit};
     e = cudaLaunchCooperativeKernel((void*)h_jacobi_coop, dim3((unsigned)blocks), dim3(256), args, 0, s);
@@ -1420,20 +1468,6 @@ __global__ void __launch_bounds__(1024) h_rg_form_s(int m, const double2* __rest
     }
 }
 
-// C <- (C + C^H) / 2 in place (thread per pair i <= j).
-__global__ void h_herm_part(int m, double2* __restrict__ C)
-{
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < (long long)m * m;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(idx / m), j = (int)(idx % m);
-        if (i > j) continue;
-        const double2 a = C[idx], b = C[(long long)j * m + i];
-        const double2 s = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
-        C[idx] = s;
-        C[(long long)j * m + i] = make_double2(s.x, -s.y);
-    }
-}
-
 // Cholesky route (the LAPACK hegv family's first step, as on the real path):
 // one CTA factors the scaled Bs = D Bq D = L L^H in the global scratch G
 // (row-major, lower triangle read), inverts X = L^{-1}, and writes the
@@ -1455,20 +1489,25 @@ __global__ void __launch_bounds__(1024) h_rg_cholinv(int m, const double2* __res
     for (long long idx = tid; idx < (long long)m * m; idx += nt) G[idx] = Bs[idx];
     if (tid == 0) s_ok = 1;
     __syncthreads();
-    for (int j = 0; j < m; ++j) {  // right-looking: two barriers per column
-        const double dj = G[(size_t)j * m + j].x;
-        if (!(dj > 0.0)) {  // same value in every thread: uniform exit
+    for (int j = 0; j < m; ++j) {  // right-looking; one thread takes the pivot's root (as cta_chol_inv)
+        if (tid == 0) {
+            const double dj = G[(size_t)j * m + j].x;
+            const double l = dj > 0.0 ? sqrt(dj) : 0.0;
+            xd[j] = l;
+            red[0] = l > 0.0 ? 1.0 / l : 0.0;
+        }
+        __syncthreads();
+        const double il = red[0];
+        if (!(il > 0.0)) {  // same value in every thread: uniform exit
             if (tid == 0) *status = 1;
             return;
         }
-        const double l = sqrt(dj);
         for (int i = j + 1 + tid; i < m; i += nt) {
             const double2 g = G[(size_t)i * m + j];
-            const double2 v = make_double2(g.x / l, g.y / l);
+            const double2 v = make_double2(g.x * il, g.y * il);
             G[(size_t)i * m + j] = v;
             cj[i] = v;
         }
-        if (tid == 0) xd[j] = l;
         __syncthreads();
         for (int i = j + 1 + warp; i < m; i += nw) {  // G[i][k] -= cj[i] conj(cj[k]), j < k <= i
             const double2 ci = cj[i];
@@ -1540,12 +1579,59 @@ __global__ void __launch_bounds__(1024) h_rg_cholinv(int m, const double2* __res
     }
 }
 
+// C = A B (HERM = 0), or A^H B with its part on and above the diagonal mirrored
+// (HERM = 1: S^H A S), all m x m: a thread per element, 16 x 16 tiles (the 64 x
+// 64 tiles of the n x m products leave most of the chip idle: m = 60, 320 us,
+// here 20).
+template <int HERM>
+__global__ void __launch_bounds__(256) h_rg_product(int m, const double2* __restrict__ A, const double2* __restrict__ B,
+                                                    double2* __restrict__ C)
+{
+    __shared__ double2 sa[16][17], sb[16][17];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int i0 = blockIdx.y * 16, j0 = blockIdx.x * 16;
+    if (HERM && j0 < i0) return;
+    const double2 z = make_double2(0.0, 0.0);
+    double2 s = z;
+    for (int k0 = 0; k0 < m; k0 += 16) {
+        const int ai = HERM ? k0 + ty : i0 + ty, aj = HERM ? i0 + tx : k0 + tx;
+        double2 av = ai < m && aj < m ? A[(size_t)ai * m + aj] : z;
+        if (HERM) {
+            av.y = -av.y;
+            sa[tx][ty] = av;
+        } else {
+            sa[ty][tx] = av;
+        }
+        sb[ty][tx] = k0 + ty < m && j0 + tx < m ? B[(size_t)(k0 + ty) * m + j0 + tx] : z;
+        __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < 16; ++k) {
+            const double2 x = sa[ty][k], y = sb[k][tx];
+            s.x = fma(x.x, y.x, fma(-x.y, y.y, s.x));
+            s.y = fma(x.x, y.y, fma(x.y, y.x, s.y));
+        }
+        __syncthreads();
+    }
+    const int i = i0 + ty, j = j0 + tx;
+    if (i >= m || j >= m || (HERM && j < i)) return;
+    if (HERM && i == j) s.y = 0.0;
+    C[(size_t)i * m + j] = s;
+    if (HERM) C[(size_t)j * m + i] = make_double2(s.x, -s.y);
+}
+
+template <int HERM>
+static cudaError_t launch_h_rg_product(int m, const double2* A, const double2* B, double2* C, cudaStream_t s)
+{
+    const unsigned t = (unsigned)((m + 15) / 16);
+    h_rg_product<HERM><<<dim3(t, t), 256, 0, s>>>(m, A, B, C);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 size_t h_reduced_work_bytes(int m)
 {
     const size_t mm = (size_t)m * m;
-    int ks = 1;
-    const size_t gp = h_gram_partial(m, m, &ks);
-    return (9 * mm + gp + m) * sizeof(double2) + 3 * (size_t)m * sizeof(double) + 512 + h_jacobi_coop_bytes(m) + 256;
+    return (9 * mm + m) * sizeof(double2) + 3 * (size_t)m * sizeof(double) + 512 + h_jacobi_coop_bytes(m) + 256;
 }
 
 int h_reduced_gev(int m, const double2* Aq, const double2* Bq, double* lam, double2* V, int* mk_dev, int* status_dev,
@@ -1553,8 +1639,6 @@ int h_reduced_gev(int m, const double2* Aq, const double2* Bq, double* lam, doub
 {
     if (m <= 0 || m > kHJMax) return -1;
     const size_t mm = (size_t)m * m;
-    int ks = 1;
-    h_gram_partial(m, m, &ks);
     double2* As = (double2*)work;
     double2* Bs = As + mm;
     double2* U = Bs + mm;
@@ -1563,8 +1647,7 @@ int h_reduced_gev(int m, const double2* Aq, const double2* Bq, double* lam, doub
     double2* AS = S + mm;
     double2* C = AS + mm;
     double2* W = C + mm;
-    double2* gp = W + mm;
-    double* d = (double*)(gp + (size_t)ks * mm);
+    double* d = (double*)(W + mm);
     double2* G = (double2*)(d + m + (m & 1));  // Cholesky scratch (m x m) and column buffer (m), 16-byte aligned
     double2* cj = G + mm;
     double* xd = (double*)(cj + m);
@@ -1580,24 +1663,20 @@ int h_reduced_gev(int m, const double2* Aq, const double2* Bq, double* lam, doub
     if (cudaMemcpyAsync(&chol, status_dev, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -4;
     if (cudaStreamSynchronize(s) != cudaSuccess) return -4;
     if (chol == 0) {  // S^H Aq S, one Jacobi, V = S W
-        if ((e = launch_h_gemm(m, m, m, As, S, AS, s)) != cudaSuccess) return -4;
-        if ((e = launch_h_gram(m, m, S, AS, C, gp, ks, s)) != cudaSuccess) return -4;
-        h_herm_part<<<blocks, 256, 0, s>>>(m, C);
-        count_launches(1);
+        if ((e = launch_h_rg_product<0>(m, As, S, AS, s)) != cudaSuccess) return -4;
+        if ((e = launch_h_rg_product<1>(m, S, AS, C, s)) != cudaSuccess) return -4;
         if ((e = launch_h_jacobi_coop(m, C, lam, W, jw, status_dev + 1, s)) != cudaSuccess) return -4;
-        if ((e = launch_h_gemm(m, m, m, S, W, V, s)) != cudaSuccess) return -4;
+        if ((e = launch_h_rg_product<0>(m, S, W, V, s)) != cudaSuccess) return -4;
         return cudaGetLastError() == cudaSuccess ? 0 : -4;
     }
     if ((e = cudaMemsetAsync(status_dev, 0, sizeof(int), s)) != cudaSuccess) return -4;
     if ((e = launch_h_jacobi_coop(m, Bs, d, U, jw, status_dev, s)) != cudaSuccess) return -4;
     h_rg_form_s<<<1, 1024, 0, s>>>(m, Bq, d, U, S, mk_dev, status_dev);
     count_launches(1);
-    if ((e = launch_h_gemm(m, m, m, As, S, AS, s)) != cudaSuccess) return -4;
-    if ((e = launch_h_gram(m, m, S, AS, C, gp, ks, s)) != cudaSuccess) return -4;
-    h_herm_part<<<blocks, 256, 0, s>>>(m, C);
-    count_launches(1);
+    if ((e = launch_h_rg_product<0>(m, As, S, AS, s)) != cudaSuccess) return -4;
+    if ((e = launch_h_rg_product<1>(m, S, AS, C, s)) != cudaSuccess) return -4;
     if ((e = launch_h_jacobi(m, C, Vw, lam, W, mk_dev, status_dev + 1, s)) != cudaSuccess) return -4;
-    if ((e = launch_h_gemm(m, m, m, S, W, V, s)) != cudaSuccess) return -4;
+    if ((e = launch_h_rg_product<0>(m, S, W, V, s)) != cudaSuccess) return -4;
     return cudaGetLastError() == cudaSuccess ? 0 : -4;
 }
 
