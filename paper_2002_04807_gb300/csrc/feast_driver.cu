@@ -1251,8 +1251,18 @@ int run_feast(const Plan& P, Bufs& B, const Csr& A, const Csr& Bm, int* fpm, dou
 static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 static constexpr int kGershBlocks = 1024;
 
-// Workspace beyond the solver's own: -A (largest mode), diag(B), Gershgorin
-// partials and a flag.
+// Subspace columns of the counting passes.
+static int extreme_count_cols(int m0) { return std::max(2, std::min(m0, 32)); }
+
+// Workspace of the search's solves and of its counting passes.
+static size_t extreme_solve_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm)
+{
+    Bufs B;
+    const Plan Ps = make_plan(n, nnz_a, nnz_b, m0, fpm), Pc = make_plan(n, nnz_a, nnz_b, extreme_count_cols(m0), fpm);
+    return std::max(carve(Ps, nullptr, B), carve(Pc, nullptr, B));
+}
+
+// Workspace beyond those: -A (largest mode), diag(B), Gershgorin partials and a flag.
 static size_t extreme_extra_bytes(int n, int nnz_a)
 {
     return al256((size_t)nnz_a * sizeof(double)) + al256((size_t)n * sizeof(double)) +
@@ -1262,10 +1272,9 @@ static size_t extreme_extra_bytes(int n, int nnz_a)
 extern "C" size_t feast_scsr_workspace_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm)
 {
     if (n <= 0 || m0 <= 0 || !fpm) return 0;
-    Plan P = make_plan(n, nnz_a, nnz_b, m0, fpm);
+    if (fpm[39] != 0) return al256(extreme_solve_bytes(n, nnz_a, nnz_b, m0, fpm)) + extreme_extra_bytes(n, nnz_a);
     Bufs B;
-    const size_t base = carve(P, nullptr, B);
-    return fpm[39] != 0 ? al256(base) + extreme_extra_bytes(n, nnz_a) : base;
+    return carve(make_plan(n, nnz_a, nnz_b, m0, fpm), nullptr, B);
 }
 
 // Smallest and largest Gershgorin bound over the rows (scaled by diag(scale)
@@ -1345,7 +1354,7 @@ static int extreme_solve(int n, int nnz_a, const int* d_ia, const int* d_ja, con
     const int M0 = *m0, k = M0 / 2, sign = fpm[39];
     Plan Pm = make_plan(n, nnz_a, d_b ? nnz_b : 0, M0, fpm);
     Bufs Bw;
-    const size_t need = carve(Pm, nullptr, Bw);
+    const size_t need = extreme_solve_bytes(n, nnz_a, d_b ? nnz_b : 0, M0, fpm);
     if (!d_work || work_bytes < al256(need) + extreme_extra_bytes(n, nnz_a)) return -120;
     char* xp = (char*)d_work + al256(need);
     double* negA = (double*)xp;
@@ -1380,7 +1389,7 @@ static int extreme_solve(int n, int nnz_a, const int* d_ia, const int* d_ja, con
     fpc[4] = 0;
     fpc[39] = 0;
     fpc[0] = 0;
-    const int sp = std::max(2, std::min(M0, 32));
+    const int sp = extreme_count_cols(M0);
     const Plan Pc = make_plan(n, nnz_a, Bm.nnz, sp, fpc);
     auto count = [&](double E, double* est) -> int {
         Bufs Bc;
