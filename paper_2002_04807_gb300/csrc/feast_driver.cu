@@ -881,7 +881,7 @@ int choose_step_a(const Plan& P, Bufs& B, cudaStream_t s)
         if (!FEAST_STEP_A_WS || P.fp64 || P.W != 32) break;
         int st4[4] = {0, 0, 0, 0};
         CK(cudaMemsetAsync(B.wstat, 0, sizeof(st4), s));
-        CK(launch_win_build(P.n, rbw, B.app, B.apk, P.fp64, B.wpk, B.whdr, B.wwin, B.wstat, s));
+        CK(launch_win_build(P.n, rbw, B.app, B.apk, P.fp64, B.wpk, B.whdr, B.wwin, B.wstat, P.W * 8, s));
         CK(cudaMemcpyAsync(st4, B.wstat, sizeof(st4), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (st4[3]) return 0;  // column indices outside [0, n): leave the matrix to the general path
@@ -909,7 +909,7 @@ int choose_step_a(const Plan& P, Bufs& B, cudaStream_t s)
         if (rbw > FEAST_WIN_RB_MAX || (rbw == 80 && P.fp64)) continue;
         int st4[4] = {0, 0, 0, 0};
         CK(cudaMemsetAsync(B.wstat, 0, sizeof(st4), s));
-        CK(launch_win_build(P.n, rbw, B.app, B.apk, P.fp64, B.wpk, B.whdr, B.wwin, B.wstat, s));
+        CK(launch_win_build(P.n, rbw, B.app, B.apk, P.fp64, B.wpk, B.whdr, B.wwin, B.wstat, 0, s));
         CK(cudaMemcpyAsync(st4, B.wstat, sizeof(st4), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (st4[3]) return 0;  // column indices outside [0, n): leave the matrix to the general path

@@ -147,7 +147,7 @@ cudaError_t launch_cast_diag(int n, const int* ia, const double* av, bool fp64, 
 // staged rows and cape entries; win_occupancy: resident CTAs per SM of that
 // step A variant (0 when it does not exist or does not fit).
 cudaError_t launch_win_build(int n, int rbw, const int* pp, const void* pk, bool fp64, void* meta, int4* hdr,
-                             int2* win, int* stat, cudaStream_t s);
+                             int2* win, int* stat, int rowb, cudaStream_t s);
 size_t win_smem_bytes(bool fp64, int W, int rbw, int capr, int cape);
 int win_occupancy(bool fp64, int W, int bmode, int rbw, size_t smem);
 cudaError_t launch_cocg_step_aw(const FilterArgs& a, bool fp64, int rbw, int k, int grid, size_t smem,

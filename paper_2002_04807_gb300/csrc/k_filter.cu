@@ -620,6 +620,7 @@ __global__ void __launch_bounds__(kThreads, FEAST_MINB_B) cocg_step_b(FilterArgs
 // publication cost (a fence and a counter) is paid per CTA, not per item.
 static constexpr int kWinGap = 4;      // column gaps up to this many rows are staged rather than split
 static constexpr int kWinKeys = 4096;  // sort capacity per row block (entries + own rows)
+static constexpr int kWinRows = 80;    // rows per block, at most
 
 __device__ __forceinline__ void mbar_init(unsigned addr, unsigned count)
 {
@@ -693,15 +694,18 @@ __device__ void block_bitonic(int* key, int P2)
 // packed entry), so one bulk copy stages it: (rbw + 4) ints -- the row
 // pointers relative to e0 (t = 0..rbw; rows past the end repeat the last), the
 // own rows' staged position at t = rbw + 1 -- then the block's entries with
-// staged positions for columns.
+// staged positions for columns.  With rowb > 0 (cocg_step_ws) rows are padded to
+// quads only, entries hold byte offsets (rowb bytes a staged row), and padding
+// points at its own row: no entry needs a test.
 template <typename PK>
-__global__ void __launch_bounds__(256) win_build(int n, int rbw, int nrbw, const int* __restrict__ pp,
+__global__ void __launch_bounds__(256) win_build(int n, int rbw, int nrbw, int rowb, const int* __restrict__ pp,
                                                  const PK* __restrict__ pk, char* __restrict__ meta,
                                                  int4* __restrict__ hdr, int2* __restrict__ win, int* stat)
 {
     __shared__ int key[kWinKeys];
     __shared__ int ws[kWinMax], we[kWinMax], wb[kWinMax];
     __shared__ int s_kv, s_nw, s_ok;
+    __shared__ int quad[kWinRows + 1];  // rowb > 0: row pointers after padding to quads
     const int tid = threadIdx.x, lane = tid & 31;
     for (int rb = blockIdx.x; rb < nrbw; rb += gridDim.x) {
         const int row0 = rb * rbw, row1 = min(n, row0 + rbw), rows = row1 - row0;
@@ -763,13 +767,24 @@ __global__ void __launch_bounds__(256) win_build(int n, int rbw, int nrbw, const
                         win[(size_t)rb * kWinMax + w] = make_int2(ws[w], we[w] - ws[w]);
                         total += we[w] - ws[w];
                     }
-                    hdr[rb] = make_int4(nw, total, own, cnt);
+                    int staged = cnt;
+                    if (rowb) {
+                        staged = 0;
+                        for (int r = 0; r <= rbw; ++r) {
+                            quad[r] = staged;
+                            if (r >= rows) continue;
+                            int len = pp[row0 + r + 1] - pp[row0 + r];
+                            if (len >= 4 && pk[pp[row0 + r + 1] - 4].x < 0) len -= 4;
+                            staged += len;
+                        }
+                    }
+                    hdr[rb] = make_int4(nw, total, own, staged);
                     int* lpp = (int*)(meta + (size_t)rb * (rbw + 4) * 4 + (size_t)e0 * sizeof(PK));
                     lpp[rbw + 1] = own;
                     lpp[rbw + 2] = 0;
                     lpp[rbw + 3] = 0;
                     atomicMax(stat + 0, total);
-                    atomicMax(stat + 1, cnt);
+                    atomicMax(stat + 1, staged);
                 } else {
                     atomicAdd(stat + 2, 1);
                 }
@@ -783,15 +798,28 @@ __global__ void __launch_bounds__(256) win_build(int n, int rbw, int nrbw, const
             char* region = meta + (size_t)rb * (rbw + 4) * 4 + (size_t)e0 * sizeof(PK);
             int* lpp = (int*)region;
             PK* lpk = (PK*)(region + (size_t)(rbw + 4) * 4);
-            for (int t = tid; t <= rbw; t += blockDim.x) lpp[t] = pp[min(row0 + t, row1)] - e0;
-            for (int t = tid; t < cnt; t += blockDim.x) {
-                PK e = pk[e0 + t];
-                if (e.x >= 0) {
-                    int w = 0;
-                    while (w + 1 < nw && e.x >= ws[w + 1]) ++w;
-                    e.x = wb[w] + e.x - ws[w];
+            if (rowb) {
+                for (int t = tid; t <= rbw; t += blockDim.x) lpp[t] = quad[t];
+                for (int r = tid >> 5; r < rows; r += blockDim.x >> 5)
+                    for (int t = lane; t < quad[r + 1] - quad[r]; t += 32) {
+                        PK e = pk[pp[row0 + r] + t];
+                        if (e.x < 0) e.x = row0 + r;
+                        int w = 0;
+                        while (w + 1 < nw && e.x >= ws[w + 1]) ++w;
+                        e.x = (wb[w] + e.x - ws[w]) * rowb;
+                        lpk[quad[r] + t] = e;
+                    }
+            } else {
+                for (int t = tid; t <= rbw; t += blockDim.x) lpp[t] = pp[min(row0 + t, row1)] - e0;
+                for (int t = tid; t < cnt; t += blockDim.x) {
+                    PK e = pk[e0 + t];
+                    if (e.x >= 0) {
+                        int w = 0;
+                        while (w + 1 < nw && e.x >= ws[w + 1]) ++w;
+                        e.x = wb[w] + e.x - ws[w];
+                    }
+                    lpk[t] = e;
                 }
-                lpk[t] = e;
             }
         }
         __syncthreads();  // shared tables are rewritten by the next row block
@@ -995,6 +1023,14 @@ __global__ void __launch_bounds__(kThreads, FEAST_AW_MINB) cocg_step_aw(FilterAr
 // mbarrier, one arrival per consumer warp), so the copies of the next item
 // are in flight while the current one computes; the consumers only wait,
 // compute and store.  Same arithmetic and partial sums as cocg_step_aw.
+// What bounds it is the compute warps' issue and their shared-memory loads, not
+// the copies (27-point 48^3, 320 columns of one node: 0.65 ms a step; keeping
+// rings of rows, 3 copied rows per row instead of 9.6, was slower, 0.75): so rows
+// are padded to quads whose padding needs no test, a thread's two rows go
+// through their quads together with the next ones loaded ahead, the warps share
+// no barrier per item, and items are counted without divisions: 0.575 ms, 57 % of
+// the shared-memory loads' rate; a contour pass of 300 columns and 16 nodes
+// 656 -> 585 ms, 27-point 96^3 (32 columns, 4 nodes) 218 -> 194.
 static constexpr int kThreadsWS = 512;          // consumer threads
 static constexpr int kMaxGroupsWS = 1024;        // column groups per problem this kernel takes
 
@@ -1002,21 +1038,6 @@ __device__ __forceinline__ void mbar_arrive(unsigned addr)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(addr) : "memory");
 }
-// OR of pred over the kThreadsWS consumer threads (named barrier 1).
-__device__ __forceinline__ bool consumers_or(bool pred)
-{
-    int r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.s32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, %2, p;\n\t"
-        "selp.s32 %0, 1, 0, q;\n}"
-        : "=r"(r)
-        : "r"((int)pred), "n"(kThreadsWS)
-        : "memory");
-    return r != 0;
-}
-
 template <typename T, int W, int BM, int RBW>
 __global__ void __launch_bounds__(kThreadsWS + 32, 1) cocg_step_ws(FilterArgs a, int kk)
 {
@@ -1039,7 +1060,7 @@ __global__ void __launch_bounds__(kThreadsWS + 32, 1) cocg_step_ws(FilterArgs a,
     const int tid = threadIdx.x, lane = tid & 31;
     const bool first = (k == 0);
     const FiltProb& P = a.probs[0];
-    const int n = P.n, nrb = P.nrb, nitems = (int)a.nitems, G = P.G;
+    const int n = P.n, nrb = P.nrb, G = P.G;
     const int* __restrict__ app = P.app;
     const unsigned cap = (unsigned)a.wcapr, cape = (unsigned)a.wcape;
     // a stage: [windows of r | own rows of p | own rows of q | entries | local row pointers]
@@ -1059,39 +1080,46 @@ __global__ void __launch_bounds__(kThreadsWS + 32, 1) cocg_step_ws(FilterArgs a,
     }
     for (int g = tid; g < G; g += blockDim.x) s_done[g] = a.grp_done[P.grp_off + g] ? 1 : 0;
     __syncthreads();  // the last CTA-wide barrier: producer and consumers part here
-    auto live_item = [&](int it) {
-        while (it < nitems && s_done[it / nrb]) it += gridDim.x;
-        return it;
+    // the CTA's next row block in a live group (the grid is at most the blocks of a group)
+    auto next = [&](int& g, int& rb) {
+        do {
+            rb += gridDim.x;
+            if (rb >= nrb) {
+                rb -= nrb;
+                ++g;
+            }
+        } while (g < G && s_done[g]);
     };
+    int g = 0, rb = blockIdx.x;
+    if (s_done[0]) next(g, rb);
 
     if (tid >= NT) {  // ---- producer warp
         // table rows of the next item, loaded one item ahead
         int4 mh = make_int4(0, 0, 0, 0);
         int2 mwv = make_int2(0, 0);
         int me0 = 0;
-        auto load_meta = [&](int it) {
-            const int rb = it % nrb;
-            mh = __ldg(a.whdr + rb);
-            mwv = __ldg(a.wwin + (size_t)rb * kWinMax + (lane & (kWinMax - 1)));
-            me0 = __ldg(app + rb * RBW);
+        auto load_meta = [&](int b) {
+            mh = __ldg(a.whdr + b);
+            mwv = __ldg(a.wwin + (size_t)b * kWinMax + (lane & (kWinMax - 1)));
+            me0 = __ldg(app + b * RBW);
         };
         int kq = 0;
-        int it = live_item(blockIdx.x);
-        if (it < nitems) load_meta(it);
-        for (; it < nitems; ++kq) {
+        if (g < G) load_meta(rb);
+        for (; g < G; ++kq) {
             const int st = kq & 1;
             const int4 h = mh;
             const int2 wv = lane < h.x ? mwv : make_int2(0, 0);
             const int e0 = me0;
-            const int nx = live_item(it + gridDim.x);
-            if (nx < nitems) load_meta(nx);
+            int ng = g, nrbk = rb;
+            next(ng, nrbk);
+            if (ng < G) load_meta(nrbk);
             if (kq >= 2) {  // the consumers released this stage (item kq - 2)
-                if (!mbar_wait(mb0 + 16 + 8 * st, ((kq >> 1) - 1) & 1, a.wlimit)) {
+                const bool ok = mbar_wait(mb0 + 16 + 8 * st, ((kq >> 1) - 1) & 1, a.wlimit);
+                if (!__all_sync(0xffffffffu, ok)) {
                     if (lane == 0) atomicExch(a.werr, 1);
-                    return;
+                    break;
                 }
             }
-            const int g = it / nrb, rb = it - g * nrb;
             const int row0 = rb * RBW, rows = min(n, row0 + RBW) - row0;
             int pos = wv.y;
 #pragma unroll
@@ -1117,8 +1145,11 @@ __global__ void __launch_bounds__(kThreadsWS + 32, 1) cocg_step_ws(FilterArgs a,
             if (lane == 31)
                 bulk_g2s(sb + lpp_off, (const char*)a.wpk + (size_t)rb * LPP * 4 + (size_t)e0 * ENTB,
                          LPP * 4u + (unsigned)h.w * ENTB, full);
-            it = nx;
+            g = ng;
+            rb = nrbk;
         }
+        // no copy lands after the CTA has left
+        for (int b = max(0, kq - 2); b < kq; ++b) mbar_wait(mb0 + 8 * (b & 1), (b >> 1) & 1, settle_limit(a.wlimit));
         return;
     }
 
@@ -1141,9 +1172,13 @@ __global__ void __launch_bounds__(kThreadsWS + 32, 1) cocg_step_ws(FilterArgs a,
                                       a.grp_count + gi, sm, red, &flag))
             finish_group_a<W>(a.cs + P.col_off + (size_t)g * W, first, red);
     };
+    // A wait that runs out sets the error flag; the warp then goes through the
+    // remaining items without waiting, computing or releasing any, so that the
+    // producer's and the other warps' waits run out too and nothing is overwritten
+    // under a reader.
+    bool good = true;
     int kq = 0;
-    for (int it = live_item(blockIdx.x); it < nitems; it = live_item(it + gridDim.x), ++kq) {
-        const int g = it / nrb, rb = it - g * nrb;
+    for (; g < G; next(g, rb), ++kq) {
         if (g != cur) {
             if (cur >= 0) publish(cur);
             cur = g;
@@ -1160,63 +1195,109 @@ __global__ void __launch_bounds__(kThreadsWS + 32, 1) cocg_step_ws(FilterArgs a,
             ql_ = (V*)a.p1 + tile + cl;
         }
         const int st = kq & 1;
-        const bool ok = mbar_wait(mb0 + 8 * st, (kq >> 1) & 1, a.wlimit);
-        if (consumers_or(!ok)) {  // flag, then leave (all consumers) once the copies in flight have landed
-            if (tid == 0) atomicExch(a.werr, 1);
-            mbar_wait(mb0 + 8 * st, (kq >> 1) & 1, settle_limit(a.wlimit));
-            mbar_wait(mb0 + 8 * (st ^ 1), ((kq + 1) >> 1) & 1, settle_limit(a.wlimit));
-            return;
-        }
-        const unsigned char* sb = base + (unsigned)st * stage_bytes;
-        const V* xs = (const V*)sb;
-        const V* ps = (const V*)(sb + p_off);
-        const V* qs = (const V*)(sb + q_off);
-        const int4* sent = (const int4*)(sb + ent_off);
-        const int* lp = (const int*)(sb + lpp_off);
         const int row0 = rb * RBW, row1 = min(n, row0 + RBW);
-        const int own0 = lp[RBW + 1];
-        T acc[3] = {T(0), T(0), T(0)};
+        T bo[RPT];  // B's diagonal, ahead of the wait
+        if (BM == 1)
 #pragma unroll
-        for (int u = 0; u < RPT; ++u) {
-            const int i = row0 + rowslot + u * RPP;
-            if (i < row1) {
-                const int c0 = lp[i - row0], c1 = lp[i - row0 + 1];
-                V ar = zero;
-                for (int c = c0; c < c1; c += kChunk) {
-                    int j[kChunk];
-                    T av[kChunk];
-                    load_chunk<T, true>(sent, c, j, av);
-                    V xv[kChunk];
-#pragma unroll
-                    for (int v = 0; v < kChunk; ++v) xv[v] = j[v] >= 0 ? xs[(size_t)j[v] * W + cl] : zero;
-#pragma unroll
-                    for (int v = 0; v < kChunk; ++v) {
-                        ar.x = fma(av[v], xv[v].x, ar.x);
-                        ar.y = fma(av[v], xv[v].y, ar.y);
-                    }
-                }
-                const V ri = xs[(size_t)(own0 + i - row0) * W + cl];
-                V bx = ri;
-                if (BM == 1) {
-                    const T b = ((const T*)P.bd)[i];
-                    bx = cmk<V>(b * ri.x, b * ri.y);
-                }
-                V pi_ = ri, qi = csub(cmul(z, bx), ar);  // (zB - A) r
-                if (use_p) {
-                    pi_ = cfma(beta, ps[(size_t)(i - row0) * W + cl], pi_);
-                    qi = cfma(beta, qs[(size_t)(i - row0) * W + cl], qi);
-                }
-                pl_[(size_t)i * W] = pi_;
-                ql_[(size_t)i * W] = qi;
-                acc[0] = fma(pi_.x, qi.x, fma(-pi_.y, qi.y, acc[0]));
-                acc[1] = fma(pi_.x, qi.y, fma(pi_.y, qi.x, acc[1]));
-                if (first) acc[2] = fma(ri.x, ri.x, fma(ri.y, ri.y, acc[2]));
-            }
+            for (int u = 0; u < RPT; ++u) bo[u] = __ldg((const T*)P.bd + min(row0 + rowslot + u * RPP, n - 1));
+        if (good && !mbar_wait(mb0 + 8 * st, (kq >> 1) & 1, a.wlimit)) {
+            atomicExch(a.werr, 1);
+            good = false;
         }
+        good = __all_sync(0xffffffffu, good);
+        if (good) {
+            const unsigned char* sb = base + (unsigned)st * stage_bytes;
+            const unsigned char* xs = sb + cl * sizeof(V);
+            const V* ps = (const V*)(sb + p_off);
+            const V* qs = (const V*)(sb + q_off);
+            const int4* sent = (const int4*)(sb + ent_off);
+            const int* lp = (const int*)(sb + lpp_off);
+            const int own0 = lp[RBW + 1];
+            T acc[3] = {T(0), T(0), T(0)};
+            // A r of the thread's rows, their quads of entries taken together, the
+            // next quads' entries loaded ahead
+            struct Quad {
+                int4 e[2];
+            };
+            V ar[RPT];
+            int c0[RPT], nch = INT_MAX;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) kahan_add(accs[q], accc[q], acc[q]);
+            for (int u = 0; u < RPT; ++u) {
+                const int t = rowslot + u * RPP;
+                ar[u] = zero;
+                c0[u] = lp[t];
+                nch = min(nch, lp[t + 1] - c0[u]);
+            }
+            auto quad = [&](int c) {
+                Quad q;
+                q.e[0] = sent[c >> 1];
+                q.e[1] = sent[(c >> 1) + 1];
+                return q;
+            };
+            auto rows_of = [&](const Quad& q, V (&xv)[4]) {
+                xv[0] = *(const V*)(xs + q.e[0].x);
+                xv[1] = *(const V*)(xs + q.e[0].z);
+                xv[2] = *(const V*)(xs + q.e[1].x);
+                xv[3] = *(const V*)(xs + q.e[1].z);
+            };
+            auto sum_of = [&](const Quad& q, const V (&xv)[4], V& sum) {
+                const T av[4] = {__int_as_float(q.e[0].y), __int_as_float(q.e[0].w), __int_as_float(q.e[1].y),
+                                 __int_as_float(q.e[1].w)};
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    sum.x = fma(av[v], xv[v].x, sum.x);
+                    sum.y = fma(av[v], xv[v].y, sum.y);
+                }
+            };
+            if (nch > 0) {
+                Quad q[RPT];
+#pragma unroll
+                for (int u = 0; u < RPT; ++u) q[u] = quad(c0[u]);
+                for (int c = 4;; c += 4) {
+                    Quad nq[RPT];
+                    V xv[RPT][4];
+#pragma unroll
+                    for (int u = 0; u < RPT; ++u) {
+                        rows_of(q[u], xv[u]);
+                        nq[u] = quad(c0[u] + min(c, nch - 4));
+                    }
+#pragma unroll
+                    for (int u = 0; u < RPT; ++u) sum_of(q[u], xv[u], ar[u]);
+                    if (c >= nch) break;
+#pragma unroll
+                    for (int u = 0; u < RPT; ++u) q[u] = nq[u];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < RPT; ++u) {
+                const int t = rowslot + u * RPP, i = row0 + t;
+                if (i < row1) {
+                    for (int c = c0[u] + nch; c < lp[t + 1]; c += 4) {
+                        const Quad q = quad(c);
+                        V xv[4];
+                        rows_of(q, xv);
+                        sum_of(q, xv, ar[u]);
+                    }
+                    const V ri = *(const V*)(xs + (unsigned)(own0 + t) * ROWB);
+                    V bx = ri;
+                    if (BM == 1) bx = cmk<V>(bo[u] * ri.x, bo[u] * ri.y);
+                    V pi_ = ri, qi = csub(cmul(z, bx), ar[u]);  // (zB - A) r
+                    if (use_p) {
+                        pi_ = cfma(beta, ps[t * W + cl], pi_);
+                        qi = cfma(beta, qs[t * W + cl], qi);
+                    }
+                    pl_[(size_t)i * W] = pi_;
+                    ql_[(size_t)i * W] = qi;
+                    acc[0] = fma(pi_.x, qi.x, fma(-pi_.y, qi.y, acc[0]));
+                    acc[1] = fma(pi_.x, qi.y, fma(pi_.y, qi.x, acc[1]));
+                    if (first) acc[2] = fma(ri.x, ri.x, fma(ri.y, ri.y, acc[2]));
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) kahan_add(accs[q], accc[q], acc[q]);
+        }
         __syncwarp();
-        if (lane == 0) mbar_arrive(mb0 + 16 + 8 * st);  // this warp is done with the stage
+        if (good && lane == 0) mbar_arrive(mb0 + 16 + 8 * st);  // this warp is done with the stage
     }
     if (cur >= 0) publish(cur);
 }
@@ -1495,15 +1576,15 @@ cudaError_t launch_cocg_step_b(const FilterArgs& a, bool fp64, int k, int grid, 
 
 // ---------------------------------------------------------------- staged-window launchers
 cudaError_t launch_win_build(int n, int rbw, const int* pp, const void* pk, bool fp64, void* meta, int4* hdr,
-                             int2* win, int* stat, cudaStream_t s)
+                             int2* win, int* stat, int rowb, cudaStream_t s)
 {
     if (n <= 0 || rbw <= 0) return cudaSuccess;
     const int nrbw = (n + rbw - 1) / rbw;
     const int grid = std::min(nrbw, num_sms() * 8);
     if (fp64)
-        win_build<int4><<<grid, 256, 0, s>>>(n, rbw, nrbw, pp, (const int4*)pk, (char*)meta, hdr, win, stat);
+        win_build<int4><<<grid, 256, 0, s>>>(n, rbw, nrbw, rowb, pp, (const int4*)pk, (char*)meta, hdr, win, stat);
     else
-        win_build<int2><<<grid, 256, 0, s>>>(n, rbw, nrbw, pp, (const int2*)pk, (char*)meta, hdr, win, stat);
+        win_build<int2><<<grid, 256, 0, s>>>(n, rbw, nrbw, rowb, pp, (const int2*)pk, (char*)meta, hdr, win, stat);
     count_launches(1);
     return cudaGetLastError();
 }
