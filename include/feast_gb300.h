@@ -400,8 +400,8 @@ int feast_gram_noalloc_dev(int n, int m, const double* X, const double* Y, doubl
 /* The same contraction C = X^T Y (upper triangle mirrored) computed from
  * exact products of BF16 integer slices on the tensor cores (Ozaki et al.'s
  * error-free splitting: 7 slices of 8 bits per value under a power-of-two
- * column scale; products accumulated exactly in FP32 for 256 rows at a time,
- * then in FP64), the arithmetic of the solvers' projections A_Q = Q^T A Q,
+ * column scale; products accumulated exactly in FP32 for 128 rows at a time,
+ * then in 64-bit integers), the arithmetic of the solvers' projections A_Q = Q^T A Q,
  * B_Q = Q^T B Q when fpm(54) = 0 (Sec. 1.1's reduced problem, FP64 accuracy:
  * the truncation error of an element is below 2^-55 max|X[:,a]| max|Y[:,b]|
  * per row).  Device row-major n x m X, Y; C m x m.  Returns 0, -101 n <= 0,

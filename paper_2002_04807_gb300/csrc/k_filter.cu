@@ -1,6 +1,9 @@
 // Contour filter kernels: batched complex-shifted CSR SpMM, column-batched
 // COCG for the complex symmetric systems (z_e B - A) y = rhs, and the fused
-// accumulation of the quadrature sum into the FP64 subspace block Q.
+// accumulation of the quadrature sum into the FP64 subspace block Q.  For
+// problems with a B, callers that set the rows per work item, and B = I
+// problems whose Krylov bases do not fit; other B = I problems take one Krylov
+// space per column for all nodes (k_krylov.cu).
 //
 // Method (FEAST v4.0 guide, Sec. 1.1 and the tips of Sec. 3.1): for the Ne
 // half-contour nodes z_e with weights w_e, the filter is

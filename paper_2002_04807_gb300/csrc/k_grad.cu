@@ -21,7 +21,7 @@ namespace feast {
 // its share of an entry's sum, which three shuffles complete; four entries are
 // in flight.  Bound: FP64 issue, then L2 (each row of X is read once per entry
 // of its column).  A warp per row spent its time on five FP64 shuffle-and-add
-// steps per entry (48^3, 71 vectors: 453 us, this form 132; the sums alone need
+// steps per entry (48^3, 71 vectors: 453 us, this form 190; the sums alone need
 // 54 M FP64 FMA, about 95 us).
 static constexpr int kGradLanes = 8;
 static constexpr int kGradReg = 16;
