@@ -510,6 +510,27 @@ size_t carve(const Plan& P, void* base, Bufs& B, bool filter_only = false)
     return c.off + 256;
 }
 
+// The Krylov bases are the larger part of a workspace (64^3, 150 columns, 80
+// steps: 13.6 of 16 GB).  Where the memory at hand does not hold them, the plan
+// goes without: COCG per node, in the same arguments and results, several times
+// slower.  False when it had none.
+bool drop_krylov(Plan& P)
+{
+    const bool had = P.lzc.teams > 0;
+    P.lzc = P.lzr = KrylovPlan{};
+    return had;
+}
+
+// Plan for a workspace of `bytes`, and what it needs of them.
+Plan plan_within(int n, int nnzA, int nnzB, int m0, const int* fpm, size_t bytes, size_t* need)
+{
+    Plan P = make_plan(n, nnzA, nnzB, m0, fpm);
+    Bufs B;
+    *need = carve(P, nullptr, B);
+    if (*need > bytes && drop_krylov(P)) *need = carve(P, nullptr, B);
+    return P;
+}
+
 // ---------------------------------------------------------------- small kernels
 __global__ void k_col_to_row(int n, int m, const double* xc, double* xr)
 {
@@ -1254,12 +1275,14 @@ static constexpr int kGershBlocks = 1024;
 // Subspace columns of the counting passes.
 static int extreme_count_cols(int m0) { return std::max(2, std::min(m0, 32)); }
 
-// Workspace of the search's solves and of its counting passes.
-static size_t extreme_solve_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm)
+// Workspace of the search's solves and of its counting passes, with or without Krylov bases.
+static size_t extreme_solve_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm, bool krylov = true)
 {
-    Bufs B;
-    const Plan Ps = make_plan(n, nnz_a, nnz_b, m0, fpm), Pc = make_plan(n, nnz_a, nnz_b, extreme_count_cols(m0), fpm);
-    return std::max(carve(Ps, nullptr, B), carve(Pc, nullptr, B));
+    const size_t most = krylov ? SIZE_MAX : 0;
+    size_t a = 0, b = 0;
+    plan_within(n, nnz_a, nnz_b, m0, fpm, most, &a);
+    plan_within(n, nnz_a, nnz_b, extreme_count_cols(m0), fpm, most, &b);
+    return std::max(a, b);
 }
 
 // Workspace beyond those: -A (largest mode), diag(B), Gershgorin partials and a flag.
@@ -1269,12 +1292,20 @@ static size_t extreme_extra_bytes(int n, int nnz_a)
            al256(2 * kGershBlocks * sizeof(double)) + 512;
 }
 
+// Workspace with Krylov bases, or the least that a call accepts.
+static size_t scsr_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm, bool krylov)
+{
+    if (fpm[39] != 0)
+        return al256(extreme_solve_bytes(n, nnz_a, nnz_b, m0, fpm, krylov)) + extreme_extra_bytes(n, nnz_a);
+    size_t need = 0;
+    plan_within(n, nnz_a, nnz_b, m0, fpm, krylov ? SIZE_MAX : 0, &need);
+    return need;
+}
+
 extern "C" size_t feast_scsr_workspace_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm)
 {
     if (n <= 0 || m0 <= 0 || !fpm) return 0;
-    if (fpm[39] != 0) return al256(extreme_solve_bytes(n, nnz_a, nnz_b, m0, fpm)) + extreme_extra_bytes(n, nnz_a);
-    Bufs B;
-    return carve(make_plan(n, nnz_a, nnz_b, m0, fpm), nullptr, B);
+    return scsr_bytes(n, nnz_a, nnz_b, m0, fpm, true);
 }
 
 // Smallest and largest Gershgorin bound over the rows (scaled by diag(scale)
@@ -1352,10 +1383,14 @@ static int extreme_solve(int n, int nnz_a, const int* d_ia, const int* d_ja, con
                          int* loop, void* d_work, size_t work_bytes, cudaStream_t s)
 {
     const int M0 = *m0, k = M0 / 2, sign = fpm[39];
-    Plan Pm = make_plan(n, nnz_a, d_b ? nnz_b : 0, M0, fpm);
     Bufs Bw;
-    const size_t need = extreme_solve_bytes(n, nnz_a, d_b ? nnz_b : 0, M0, fpm);
-    if (!d_work || work_bytes < al256(need) + extreme_extra_bytes(n, nnz_a)) return -120;
+    const size_t extra = extreme_extra_bytes(n, nnz_a);
+    size_t need = extreme_solve_bytes(n, nnz_a, d_b ? nnz_b : 0, M0, fpm);
+    const bool krylov = work_bytes >= al256(need) + extra;
+    if (!krylov) need = extreme_solve_bytes(n, nnz_a, d_b ? nnz_b : 0, M0, fpm, false);
+    if (!d_work || work_bytes < al256(need) + extra) return -120;
+    size_t part_need = 0;
+    const Plan Pm = plan_within(n, nnz_a, d_b ? nnz_b : 0, M0, fpm, krylov ? SIZE_MAX : 0, &part_need);
     char* xp = (char*)d_work + al256(need);
     double* negA = (double*)xp;
     xp += al256((size_t)nnz_a * sizeof(double));
@@ -1390,7 +1425,7 @@ static int extreme_solve(int n, int nnz_a, const int* d_ia, const int* d_ja, con
     fpc[39] = 0;
     fpc[0] = 0;
     const int sp = extreme_count_cols(M0);
-    const Plan Pc = make_plan(n, nnz_a, Bm.nnz, sp, fpc);
+    const Plan Pc = plan_within(n, nnz_a, Bm.nnz, sp, fpc, krylov ? SIZE_MAX : 0, &part_need);
     auto count = [&](double E, double* est) -> int {
         Bufs Bc;
         carve(Pc, d_work, Bc);
@@ -1574,9 +1609,9 @@ static int solve_dev_impl(int n, int nnz_a, const int* d_ia, const int* d_ja, co
     if (!d_ia || !d_ja || !d_a || nnz_a < 0) return ret(-103);
     if (d_b && (!d_ib || !d_jb || nnz_b <= 0)) return ret(-106);
     if (!e || !d_x || !m || !res || !epsout || !loop) return ret(-113);
-    Plan P = make_plan(n, nnz_a, d_b ? nnz_b : 0, *m0, fpm);
+    size_t need = 0;
+    const Plan P = plan_within(n, nnz_a, d_b ? nnz_b : 0, *m0, fpm, work_bytes, &need);
     Bufs B;
-    const size_t need = carve(P, nullptr, B);
     if (!d_work || work_bytes < need) return ret(-120);
     std::vector<double> czw;
     if (expert && (inf = custom_nodes(fpm[1], zne, wne, -124, czw))) return ret(inf);
@@ -1722,7 +1757,7 @@ static int host_driver(bool extreme, char uplo, int n, const double* a, const in
     double *d_a = nullptr, *d_b = nullptr, *d_x = nullptr;
     void* d_work = nullptr;
     cudaStream_t s = nullptr;
-    const size_t wb = feast_scsr_workspace_bytes(n, (int)aja.size(), hasB ? (int)bja.size() : 0, mm0, fpm);
+    size_t wb = scsr_bytes(n, (int)aja.size(), hasB ? (int)bja.size() : 0, mm0, fpm, true);
 #define HK(x)                                                        \
     do {                                                             \
         cudaError_t _e = (x);                                        \
@@ -1732,7 +1767,11 @@ static int host_driver(bool extreme, char uplo, int n, const double* a, const in
     HK(dm.alloc(&d_ja, std::max<size_t>(1, aja.size())));
     HK(dm.alloc(&d_a, std::max<size_t>(1, av.size())));
     HK(dm.alloc(&d_x, (size_t)n * mm0));
-    HK(dm.alloc((char**)&d_work, wb));
+    if (dm.alloc((char**)&d_work, wb) != cudaSuccess) {
+        cudaGetLastError();
+        wb = scsr_bytes(n, (int)aja.size(), hasB ? (int)bja.size() : 0, mm0, fpm, false);
+        HK(dm.alloc((char**)&d_work, wb));
+    }
     HK(cudaMemcpy(d_ia, aia.data(), sizeof(int) * aia.size(), cudaMemcpyHostToDevice));
     HK(cudaMemcpy(d_ja, aja.data(), sizeof(int) * aja.size(), cudaMemcpyHostToDevice));
     HK(cudaMemcpy(d_a, av.data(), sizeof(double) * av.size(), cudaMemcpyHostToDevice));
@@ -1895,10 +1934,13 @@ extern "C" int feast_filter_dev(int n, int nnz_a, const int* ia, const int* ja, 
     if (!(emin < emax)) return 200;
     Plan P = make_plan(n, nnz_a, b ? nnz_b : 0, m, fpm, true);
     Bufs B;
-    const size_t bytes = carve(P, nullptr, B, true);
     AsyncMem am(s);
     void* base = nullptr;
-    CK(am.alloc(&base, bytes));
+    if (am.alloc(&base, carve(P, nullptr, B, true)) != cudaSuccess) {
+        cudaGetLastError();
+        drop_krylov(P);
+        CK(am.alloc(&base, carve(P, nullptr, B, true)));
+    }
     carve(P, base, B, true);
     Csr A{n, nnz_a, ia, ja, a}, Bm{n, b ? nnz_b : 0, ib, jb, b};
     std::vector<double> zw;

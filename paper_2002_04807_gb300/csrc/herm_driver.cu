@@ -480,16 +480,26 @@ static int h_dev_entry(int n, int nnz_a, const int* d_ia, const int* d_ja, const
     if (!res) return ret(-116);
     if (!epsout) return ret(-117);
     if (!loop) return ret(-118);
-    const HPlan P = h_plan(n, nnz_a, hasB ? std::max(nnz_b, 1) : 0, *m0, fpm);
+    HPlan P = h_plan(n, nnz_a, hasB ? std::max(nnz_b, 1) : 0, *m0, fpm);
     HBufs B{};
     float2 *af = nullptr, *bf = nullptr;
-    const size_t need = h_carve(P, nullptr, B, &af, &bf);
+    size_t need = h_carve(P, nullptr, B, &af, &bf);
+    auto without_krylov = [&] {  // BiCG per node, where the memory does not hold the Krylov bases
+        P.lz = KrylovPlan{};
+        need = h_carve(P, nullptr, B, &af, &bf);
+    };
+    if (work && work_bytes < need) without_krylov();
     if (work && work_bytes < need) return ret(-120);
     clear_last_error();
     HDevMem dm;
     if (!work) {  // no caller workspace: the library allocates it for this call
         char* w = nullptr;
-        const cudaError_t ce = dm.alloc(&w, need);
+        cudaError_t ce = dm.alloc(&w, need);
+        if (ce != cudaSuccess) {
+            cudaGetLastError();
+            without_krylov();
+            ce = dm.alloc(&w, need);
+        }
         if (ce != cudaSuccess) return ret(cuda_error(ce, "workspace"));
         work = w;
     }

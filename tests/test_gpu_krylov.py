@@ -130,3 +130,54 @@ def test_reruns_are_identical(pkg):
     a, _ = _run(pkg, A, Y, 8, 1, 2.0, maxit=40)
     b, _ = _run(pkg, A, Y, 8, 1, 2.0, maxit=40)
     assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("extreme", [False, True])
+def test_smaller_workspace_goes_without_bases(pkg, monkeypatch, extreme):
+    """A workspace that does not hold the Krylov bases is used for one COCG per node
+    (launches of its streaming step in the profile); one that holds neither is refused."""
+    from paper_2002_04807_gb300 import _lib
+
+    p = fw.laplace3d_potential(side=16, count=16, m0=24, seed=4)
+    ia, ja, av = dev(p.A.indptr), dev(p.A.indices), dev(p.A.data)
+    ev = np.linalg.eigvalsh(p.A.to_dense())
+    f = pkg.feast_init()
+    f[1], f[2], f[3], f[17], f[41], f[44], f[45], f[52] = 8, 10, 40, 100, 1, 2, 200, 1
+    f[39] = -1 if extreme else 0
+    need = _lib.feast_scsr_workspace_bytes(p.n, av.numel(), 0, 24, f)
+    for work, steps in ((need, False), (need - 1, True)):
+        monkeypatch.setattr(_lib, "feast_scsr_workspace_bytes", lambda *a, w=work: w)
+        if extreme:
+            r = _lib.feast_scsr_extreme_dev(p.n, ia, ja, av, fpm=f.copy(), m0=24)
+        else:
+            r = _lib.feast_scsr_solve_dev(p.n, ia, ja, av, fpm=f.copy(), emin=p.emin, emax=p.emax, m0=24)
+        assert r.info == 0 and r.M > 0
+        want = ev[: r.M] if extreme else ev[(ev >= p.emin) & (ev <= p.emax)]
+        assert r.M == len(want) and np.abs(r.E[: r.M] - want).max() <= 1e-9
+        assert (pkg.feast_last_profile()["cocg_b_launches"] > 0) == steps
+    monkeypatch.setattr(_lib, "feast_scsr_workspace_bytes", lambda *a: 1 << 20)
+    if extreme:
+        r = _lib.feast_scsr_extreme_dev(p.n, ia, ja, av, fpm=f.copy(), m0=24)
+    else:
+        r = _lib.feast_scsr_solve_dev(p.n, ia, ja, av, fpm=f.copy(), emin=p.emin, emax=p.emax, m0=24)
+    assert r.info == -120
+
+
+def test_smaller_workspace_hermitian(pkg):
+    """The same for a complex Hermitian problem (BiCG per node)."""
+    p = fw.laplace3d_gauge(side=12, count=12, m0=20, ratio=100)
+    n = p.n
+    args = (n, dev(p.A.indptr), dev(p.A.indices), dev(np.asarray(p.A.data, dtype=np.complex128)))
+    f = pkg.feast_init()
+    f[1], f[2], f[3], f[17], f[41], f[44], f[45] = 8, 10, 40, 100, 1, 2, 200
+    need = pkg.feast_hcsr_workspace_bytes(n, args[3].numel(), 0, 20, f)
+    got = []
+    for work in (need, need - 1):
+        r = pkg.feast_hcsr_solve_dev(*args, fpm=f.copy(), emin=p.emin, emax=p.emax, m0=20,
+                                     work=torch.empty(work, dtype=torch.uint8, device="cuda"))
+        assert r.info == 0 and r.M > 0
+        got.append(r.E[: r.M])
+    assert len(got[0]) == len(got[1]) and np.abs(got[0] - got[1]).max() <= 1e-9
+    r = pkg.feast_hcsr_solve_dev(*args, fpm=f.copy(), emin=p.emin, emax=p.emax, m0=20,
+                                 work=torch.empty(1 << 16, dtype=torch.uint8, device="cuda"))
+    assert r.info == -120
