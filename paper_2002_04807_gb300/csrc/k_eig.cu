@@ -79,9 +79,9 @@ __device__ __forceinline__ int rr_player(int slot, int r, int mp)
 // Rotation of the pair (p, q): t near the smaller root of
 // f(t) = b t^2 + d t - b, b = apq, d = aqq - app (scaled near 1): the root in
 // single precision and one Newton step in FP64 (about 1e-13 of b is left), and
-// c = 1 / sqrt(1 + t^2), s = t c to FP64 (a single-precision seed and two
-// Newton steps), so the rotation is orthogonal to rounding although it leaves
-// -c^2 f(t) in the place of apq.  Fifteen FP64 operations instead of two
+// c = 1 / sqrt(1 + t^2), s = t c to FP64 (a single-precision seed and the
+// first two terms of the binomial series), so the rotation is orthogonal to rounding although it leaves
+// -c^2 f(t) in the place of apq.  Twelve FP64 operations instead of two
 // divisions and two square roots, which held every round up while all CTAs
 // computed all angles.
 __device__ __forceinline__ void jac_rotation(double d, double b, double& c, double& s, double& t)
@@ -91,11 +91,10 @@ __device__ __forceinline__ void jac_rotation(double d, double b, double& c, doub
     t = (double)x;
     t = fma(-fma(fma(b, t, d), t, -b), (double)(1.0f / fmaf(2.0f * bf, x, df)), t);
     const double y = fma(t, t, 1.0);
-    double r = (double)rsqrtf((float)y);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) r = r * fma(-0.5 * y * r, r, 1.5);
-    c = r;
-    s = t * r;
+    const double r = (double)rsqrtf((float)y);
+    const double e = fma(-y * r, r, 1.0);
+    c = fma(r * e, fma(0.375, e, 0.5), r);
+    s = t * c;
 }
 
 // Cyclic Jacobi of one matrix by a team of CTAs, one barrier per round: every
@@ -104,11 +103,13 @@ __device__ __forceinline__ void jac_rotation(double d, double b, double& c, doub
 // blocks from the current copy of A into the other copy, so no CTA writes what
 // another still reads.  Of two blocks that mirror each other one is computed
 // and written twice.  A round is a chain of latencies (at m = 150 with 90 CTAs
-// 1.3 us of loads and angles, 1.2 the blocks, 0.4 V, 1.7 the barrier; FP64
+// 1.2 us of loads and angles, 1.2 the blocks, 1.7 the barrier; FP64
 // operations take some 100 cycles one after the other): the entries of a
 // thread's first block and of its first pair of V load together with those of
-// the angles, and its place in the round's table is worked out once.  7.7 us a
-// round before, 4.6 now.  A sweep ends with a look for
+// the angles, its place in the round's table is worked out once, and V, whose
+// rows belong to one CTA each, is updated between the CTA's arrival at the
+// barrier and its wait.  7.7 us a round before, 4.6 with V ahead of the barrier
+// (m = 150: 4.79 ms of a reduced problem), 4.1 now (4.44).  A sweep ends with a look for
 // entries above the threshold, so no whole sweep is spent on finding none.
 // Rotation tables in dynamic shared memory: c, s, t (doubles), p, q (ints).
 // Tasks: `one` (pr == nullptr) or the batch's active problems in turn.
@@ -187,8 +188,11 @@ __global__ void __launch_bounds__(kEigThreads) jacobi_team(JacArgs a)
         };
         // a thread's first block (k, l) and first pair of a row of V
         int k0 = 0, l0 = 0;
-        const bool has = block(gtid, k0, l0), hasv = gtid < m * half;
-        const int i0 = gtid / half, kv0 = gtid - i0 * half;
+        const bool has = block(gtid, k0, l0);
+        // V's rows go to the CTAs in turn: no other CTA reads them before the end
+        const int vitems = cta < m ? ((m - 1 - cta) / nc + 1) * half : 0;
+        const bool hasv = (int)threadIdx.x < vitems;
+        const int i0 = cta + (int)threadIdx.x / half * nc, kv0 = (int)threadIdx.x % half;
         int sweep = 0;
         for (; sweep < kMaxSweeps && mp >= 2; ++sweep) {
             for (int r = 0; r < mp - 1; ++r) {
@@ -268,20 +272,22 @@ __global__ void __launch_bounds__(kEigThreads) jacobi_team(JacArgs a)
                         nxt[(size_t)qq * m + q] = z11;
                     }
                 }
-                for (int idx = gtid; idx < m * half; idx += gsz) {
-                    const int i = idx == gtid ? i0 : idx / half, k = idx == gtid ? kv0 : idx - i * half;
+                team_arrive(&w->count, target, nc);
+                for (int idx = threadIdx.x; idx < vitems; idx += blockDim.x) {  // behind the other CTAs' arrivals
+                    const bool own = idx == (int)threadIdx.x;
+                    const int i = own ? i0 : cta + idx / half * nc, k = own ? kv0 : idx % half;
                     const double sk = rs[k];
                     if (sk == 0.0) continue;
                     const double ck = rc[k];
                     const int p = rp[k], q = rq[k];
-                    if (idx != gtid) {
+                    if (!own) {
                         vp = __ldcg(V + (size_t)i * m + p);
                         vq = __ldcg(V + (size_t)i * m + q);
                     }
                     V[(size_t)i * m + p] = ck * vp - sk * vq;
                     V[(size_t)i * m + q] = sk * vp + ck * vq;
                 }
-                if (!team_sync(&w->count, target, nc, &w->err, a.limit)) return;
+                if (!team_wait(&w->count, target, nc, &w->err, a.limit)) return;
                 double* tmp = cur;
                 cur = nxt;
                 nxt = tmp;

@@ -1150,13 +1150,11 @@ struct HJWork {
     int again[2];  // a sweep left an entry above the threshold
 };
 
-// 1 / sqrt(y) for y within single-precision range: a seed and two Newton steps.
+// 1 / sqrt(y) for y within single-precision range: a seed and the first two terms of the binomial series.
 __device__ __forceinline__ double h_rsqrt(double y)
 {
-    double r = (double)rsqrtf((float)y);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) r = r * fma(-0.5 * y * r, r, 1.5);
-    return r;
+    const double r = (double)rsqrtf((float)y), e = fma(-y * r, r, 1.0);
+    return fma(r * e, fma(0.375, e, 0.5), r);
 }
 
 __global__ void __launch_bounds__(256) h_jacobi_coop(int m, double2* __restrict__ A, double2* __restrict__ A2,
@@ -1215,8 +1213,11 @@ __global__ void __launch_bounds__(256) h_jacobi_coop(int m, double2* __restrict_
     double2* nxt = A2;
     const double2 z0 = make_double2(0.0, 0.0);
     int k0 = 0, l0 = 0;
-    const bool has = block(gtid, k0, l0), hasv = gtid < m * half;
-    const int i0 = gtid / half, kv0 = gtid - i0 * half;
+    const bool has = block(gtid, k0, l0);
+    // V's rows go to the CTAs in turn: no other CTA reads them before the end
+    const int cta = blockIdx.x, vitems = cta < m ? ((m - 1 - cta) / nc + 1) * half : 0;
+    const bool hasv = (int)threadIdx.x < vitems;
+    const int i0 = cta + (int)threadIdx.x / half * nc, kv0 = (int)threadIdx.x % half;
     int sweep = 0;
     bool more = m > 1;
     while (more && sweep < kHJSweeps) {
@@ -1320,14 +1321,16 @@ __global__ void __launch_bounds__(256) h_jacobi_coop(int m, double2* __restrict_
                 if (qv) put(q, pp, make_double2(cl * y10.x - sl * ey11.x, cl * y10.y - sl * ey11.y));
                 if (qv && qqv) put(q, qq, make_double2(sl * y10.x + cl * ey11.x, sl * y10.y + cl * ey11.y));
             }
-            for (int idx = gtid; idx < m * half; idx += gsz) {  // V <- V J
-                const int i = idx == gtid ? i0 : idx / half, k = idx == gtid ? kv0 : idx - i * half;
+            team_arrive(&w->count, target, nc);
+            for (int idx = threadIdx.x; idx < vitems; idx += blockDim.x) {  // V <- V J, behind the other CTAs' arrivals
+                const bool own = idx == (int)threadIdx.x;
+                const int i = own ? i0 : cta + idx / half * nc, k = own ? kv0 : idx % half;
                 const double sk = s_s[k];
                 if (sk == 0.0) continue;
                 const double ck = s_c[k];
                 const double2 ec = make_double2(s_e[k].x, -s_e[k].y);
                 const int p = s_p[k], q = s_q[k];
-                if (idx != gtid) {
+                if (!own) {
                     vp = __ldcg(Vw + (size_t)i * m + p);
                     vq = __ldcg(Vw + (size_t)i * m + q);
                 }
@@ -1335,7 +1338,7 @@ __global__ void __launch_bounds__(256) h_jacobi_coop(int m, double2* __restrict_
                 Vw[(size_t)i * m + p] = make_double2(ck * vp.x - sk * evq.x, ck * vp.y - sk * evq.y);
                 Vw[(size_t)i * m + q] = make_double2(sk * vp.x + ck * evq.x, sk * vp.y + ck * evq.y);
             }
-            if (!team_sync(&w->count, target, nc, &w->err, limit)) return;
+            if (!team_wait(&w->count, target, nc, &w->err, limit)) return;
             double2* tmp = cur;
             cur = nxt;
             nxt = tmp;
