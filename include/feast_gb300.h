@@ -245,7 +245,8 @@ typedef struct feast_result {
 /* Many independent problems of uneven size and interval solved together (the
  * guide's first level of parallelism, Sec. 1.1: separate search intervals).
  * One set of filter launches serves all unfinished problems; the COCG steps
- * and the batched Rayleigh-Ritz sequence replay as captured CUDA graphs; the
+ * replay as a captured CUDA graph (problems with B; without, a pass is one
+ * launch per class of sizes); the
  * rows per work item of the gathering step are picked by timing a few
  * choices on the batch (cached per size class) unless fpm(51) sets them.
  * The contour nodes come from fpm(2), fpm(18) and each problem's interval;
@@ -257,7 +258,9 @@ typedef struct feast_result {
 int feast_scsr_solve_batched(int np, const feast_problem* probs, int* fpm, feast_result* out);
 
 /* Device workspace, in bytes, that feast_scsr_solve_dev needs for this
- * problem size and these parameters (fpm(2), fpm(42), fpm(50), fpm(51)). */
+ * problem size and these parameters (fpm(2), fpm(42), fpm(46), fpm(50), fpm(51)).
+ * Without B most of it holds the Krylov bases; a smaller workspace that holds
+ * the vectors of one COCG per node is used for that, several times slower. */
 size_t feast_scsr_workspace_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm);
 
 /* Same as feast_scsr_solve with the matrices and X already on the device.

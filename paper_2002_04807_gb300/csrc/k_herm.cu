@@ -1140,7 +1140,7 @@ cudaError_t launch_h_jacobi(int m, double2* A, double2* Vw, double* lam, double2
 // and one Newton step, and -c^2 f(t), about 1e-13 of a_pq, is what is left in
 // the place of a_pq.  hypot, four divisions and two square roots per angle in
 // every CTA, and a last sweep that found nothing, took 3.7 ms at m = 60, now
-// 2.3.  The barrier gives up after the wait limit: every CTA returns and
+// 2.2.  The barrier gives up after the wait limit: every CTA returns and
 // err is set.
 struct HJWork {
     unsigned count;  // barrier arrivals
