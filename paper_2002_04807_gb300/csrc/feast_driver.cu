@@ -378,6 +378,7 @@ struct Bufs {
     KrylovArgs lz = {};
     const KrylovPlan* lzp = nullptr;  // the form chosen for the matrix
     char* lzmem = nullptr;
+    double* lzmax = nullptr;  // [0] largest |entry| of A, [1] (int) rows beyond eight entries
 };
 
 size_t cplx_bytes(const Plan& P) { return P.fp64 ? 16 : 8; }
@@ -475,6 +476,7 @@ size_t carve(const Plan& P, void* base, Bufs& B, bool filter_only = false)
         const size_t bc = krylov_layout(P.lzc, nullptr, t);
         const size_t br = P.lzr.teams > 0 ? krylov_layout(P.lzr, nullptr, t) : 0;
         B.lzmem = c.take<char>(std::max(bc, br));
+        B.lzmax = c.take<double>(2);
     }
     if (P.win && !lz) {
         const size_t nrb32 = ((size_t)P.n + 31) / 32;
@@ -846,7 +848,8 @@ int filter_pass(const Plan& P, Bufs& B, int rii, const double* R, const double* 
 // entries (padded row pointers computed on the host from a copy of ia), or,
 // when allow_diag and the matrix is diagonal, just its diagonal values.
 // *mode: 1 diagonal, 2 packed.
-int pack_matrix(const Csr& M, bool fp64, bool allow_diag, int* d_pp, void* d_pk, void* d_bd, int* mode, cudaStream_t s)
+int pack_matrix(const Csr& M, bool fp64, bool allow_diag, int* d_pp, void* d_pk, void* d_bd, int* mode, cudaStream_t s,
+                const double* amax = nullptr)
 {
     const int n = M.n;
     std::vector<int> ia(n + 1);
@@ -870,7 +873,7 @@ int pack_matrix(const Csr& M, bool fp64, bool allow_diag, int* d_pp, void* d_pk,
         pp[i + 1] = pp[i] + (len + 7) / 8 * 8;
     }
     CK(cudaMemcpyAsync(d_pp, pp.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s));
-    CK(launch_pack_csr(n, M.ia, M.ja, M.v, d_pp, fp64, d_pk, s));
+    CK(launch_pack_csr(n, M.ia, M.ja, M.v, d_pp, fp64, d_pk, s, amax));
     CK(cudaStreamSynchronize(s));  // pp is a host temporary
     *mode = 2;
     return 0;
@@ -963,10 +966,11 @@ int setup_krylov(const Plan& P, Bufs& B, const Csr& A, cudaStream_t s)
     B.wrb = 0;
     B.wws = false;
     int wide = 1;
-    if ((long long)A.nnz <= 8LL * A.n) {
-        int* d_wide = (int*)B.lzmem;
-        CK(cudaMemsetAsync(d_wide, 0, sizeof(int), s));
-        CK(launch_krylov_scan(A.n, A.ia, A.ja, d_wide, s));
+    int* d_wide = (int*)(B.lzmax + 1);
+    const bool few = (long long)A.nnz <= 8LL * A.n;
+    CK(cudaMemsetAsync(B.lzmax, 0, 2 * sizeof(double), s));
+    CK(launch_krylov_scan(A.n, A.ia, few ? A.ja : nullptr, d_wide, (size_t)A.nnz, A.v, B.lzmax, s));
+    if (few) {
         CK(cudaMemcpyAsync(&wide, d_wide, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
     }
@@ -975,11 +979,11 @@ int setup_krylov(const Plan& P, Bufs& B, const Csr& A, cudaStream_t s)
     B.lz.one_chunk = wide ? 0 : 1;
     B.RB = B.lzp->resident ? 64 : 256;
     if (!wide) {
-        CK(launch_krylov_pack(A.n, B.lzp->rpc, A.ia, A.ja, A.v, P.fp64, B.apk, s));
+        CK(launch_krylov_pack(A.n, B.lzp->rpc, A.ia, A.ja, A.v, B.lzmax, P.fp64, B.apk, s));
         return 0;
     }
     int amode = 0;
-    return pack_matrix(A, P.fp64, false, B.app, B.apk, nullptr, &amode, s);
+    return pack_matrix(A, P.fp64, false, B.app, B.apk, nullptr, &amode, s, B.lzmax);
 }
 
 int setup_filter(const Plan& P, Bufs& B, const Csr& A, const Csr& Bm, const std::vector<double>& zw,
@@ -1029,6 +1033,7 @@ int setup_filter(const Plan& P, Bufs& B, const Csr& A, const Csr& Bm, const std:
     fp.zw = B.zw;
     fp.lam = lam;
     fp.mk = mk;
+    fp.amax = B.lzmax;
     fp.ne = P.ne;
     fp.active = 1;
     CK(cudaMemcpyAsync(B.probs, &fp, sizeof(fp), cudaMemcpyHostToDevice, s));
@@ -2470,6 +2475,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         (void)bump.take<char>(lz_bytes);
         (void)bump.take<int2>(max_units);
         (void)bump.take<char>(jacobi_batch_bytes(np));
+        (void)bump.take<double>(np);
         if (pass == 0) {
             cudaError_t e = dm.alloc(&base, bump.off + 4096);
             if (e != cudaSuccess) return cuda_fail(e, "batched workspace");
@@ -2524,6 +2530,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
     char* d_lz = bump.take<char>(lz_bytes);
     int2* d_units = bump.take<int2>(max_units);
     char* d_jwork = bump.take<char>(jacobi_batch_bytes(np));
+    double* d_amax = bump.take<double>(np);  // largest |entry| of every A
     std::vector<int> rpc(np, 0);  // rows per CTA of each problem's resident form
     for (Kind& kd : kinds) {
         krylov_layout(kd.plan, d_lz, kd.args);
@@ -2540,6 +2547,12 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         long long oa = 0, onz = 0, ob = 0, onzb = 0, opp = 0, opk = 0, oppb = 0, opkb = 0;
         std::vector<double> zw_all((size_t)np * ne * 4);
         std::vector<int> hasx(np, 0);
+        std::vector<double> amax(np, 0.0);
+        if (lz) {
+            for (int p = 0; p < np; ++p)
+                for (const double v : av[p]) amax[p] = std::max(amax[p], std::fabs(v));
+            CK(cudaMemcpyAsync(d_amax, amax.data(), sizeof(double) * np, cudaMemcpyHostToDevice, s));
+        }
         for (int p = 0; p < np; ++p) {
             const int n = probs[p].n;
             CK(cudaMemcpyAsync(d_ia + oa, aia[p].data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s));
@@ -2551,7 +2564,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
             f.ja = b.ja = d_ja + onz;
             f.av = b.av = d_a + onz;
             if (lz) {
-                CK(launch_krylov_pack(n, rpc[p], d_ia + oa, d_ja + onz, d_a + onz, fp64, d_apk + opk * pkz, s));
+                CK(launch_krylov_pack(n, rpc[p], d_ia + oa, d_ja + onz, d_a + onz, d_amax + p, fp64, d_apk + opk * pkz, s));
             } else {
                 // padded chunk pointers from the host copy
                 std::vector<int> pp(n + 1, 0);
@@ -2596,6 +2609,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
             f.zw = d_zw + (size_t)p * ne * 4;
             f.lam = d_lam + b.l_off;
             f.mk = d_mk + p;
+            f.amax = d_amax + p;
             if (probs[p].x0) {
                 hasx[p] = 1;
                 CK(cudaMemcpyAsync(d_xc + b.q_off, probs[p].x0, sizeof(double) * (size_t)n * probs[p].m0,

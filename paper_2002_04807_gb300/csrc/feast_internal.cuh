@@ -5,6 +5,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <cmath>
+
 namespace feast {
 
 // ---------------------------------------------------------------- complex helpers
@@ -51,6 +53,7 @@ struct FiltProb {
     const double* zw;   // Ne nodes and weights, [Ne][4] = (Re z, Im z, Re w, Im w)
     const double* lam;  // Ritz values of the previous Rayleigh-Ritz step [m0]
     const int* mk;      // live subspace columns (device), or nullptr for m0
+    const double* amax; // largest |entry| of A (device): the Krylov filter's scale
     int ne;             // number of contour nodes
     int active;         // 0: problem finished, its items are skipped
 };
@@ -133,8 +136,9 @@ cudaError_t launch_shifted_spmm(const FilterArgs& a, bool fp64, int grid, cudaSt
 cudaError_t launch_cast_values(const double* src, float* dst, long long n, cudaStream_t s);
 cudaError_t launch_advance(int* kdev, cudaStream_t s);
 cudaError_t launch_fold_dq(const FilterArgs& a, long long max_total, bool fp64, cudaStream_t s);
+// amax, if given: the values are multiplied by krylov_scale(*amax)
 cudaError_t launch_pack_csr(int n, const int* ia, const int* ja, const double* av, const int* pp, bool fp64, void* out,
-                            cudaStream_t s);
+                            cudaStream_t s, const double* amax = nullptr);
 cudaError_t launch_cast_diag(int n, const int* ia, const double* av, bool fp64, void* out, cudaStream_t s);
 // Staged-window gather (k_filter.cu).  win_build: for every row block of rbw
 // rows of the packed matrix (pp, pk), its windows (hdr, win) and, in one
@@ -185,7 +189,7 @@ struct KrylovArgs {
     void* part;         // [team][2][nc][cols] partial sums (8 bytes)
     double* coef;       // [team][2][maxit + 2][cols] alpha_j, beta_{j+1}
     void* g;            // [team][maxit][cols] combination coefficients (filter precision)
-    float4* pair;       // [team][ne][cols]
+    void* pair;         // [team][ne][cols] pivot and residual of every pair (LzPair)
     int* kstop;         // [team][ne][cols]
     double2* piv;       // [team][cols][maxit][nl]
     unsigned* bar;      // [team][32], zeroed
@@ -205,12 +209,23 @@ constexpr double kKrylovBytes = 64e9;
 KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes);
 KrylovPlan krylov_plan_set(bool fp64, int np, const int* n, const int* m, int ne, int maxit, double max_bytes);
 int krylov_rows(int n, int nc);  // rows per CTA of the resident form
+// Power of two by which the Krylov filter multiplies A and the shifts, so that
+// the steps run on entries near 1 whatever the size of A's (amax: the largest).
+__host__ __device__ inline double krylov_scale(double amax)
+{
+    if (!(amax > 0.0) || !(amax < 1.7e308)) return 1.0;
+    const int e = ilogb(amax);
+    return ldexp(1.0, e < -1000 ? 1000 : -e);
+}
 size_t krylov_layout(const KrylovPlan& k, char* base, KrylovArgs& a);
-cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, cudaStream_t s);
-cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, bool fp64, void* out,
+// amax (zeroed): the largest |v| of count values; wide (zeroed), unless ja is
+// null: set when a row needs more than eight packed entries.
+cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, size_t count, const double* v, double* amax,
                                cudaStream_t s);
-cudaError_t launch_krylov_pack_hermitian(int n, const int* ia, const int* ja, const double2* av, const int* pp, bool fp64,
-                                         void* out, cudaStream_t s);
+cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, const double* amax, bool fp64,
+                               void* out, cudaStream_t s);
+cudaError_t launch_krylov_pack_hermitian(int n, const int* ia, const int* ja, const double2* av, const int* pp,
+                                         const double* amax, bool fp64, void* out, cudaStream_t s);
 cudaError_t launch_krylov_filter(const KrylovArgs& a, const KrylovPlan& p, bool fp64, cudaStream_t s);
 
 // persistent grid size of the COCG kernels: SMs x resident CTAs per SM

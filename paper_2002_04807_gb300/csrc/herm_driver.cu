@@ -134,6 +134,7 @@ struct HBufs {
     int* lzpp;          // packed rows of the real operator
     void* lzpk;
     int* lzit;          // steps per node batch
+    double* lzmax;      // largest component of A's entries
     void* ozw;          // workspace of the sliced products (nullptr: FP64 DMMA products)
 };
 
@@ -308,6 +309,7 @@ size_t h_carve(const HPlan& P, void* base, HBufs& B, float2** af, float2** bf)
         B.lzpp = c.take<int>(2 * (size_t)P.n + 1);
         B.lzpk = c.take<char>((4 * (size_t)P.nnz_a + 14 * (size_t)P.n) * (P.fp64 ? 16 : 8));
         B.lzit = c.take<int>(P.ne);
+        B.lzmax = c.take<double>(1);
     }
     void** fv[6] = {&B.fa.r, &B.fa.rh, &B.fa.p, &B.fa.ph, &B.fa.q, &B.fa.qh};
     for (void** v : fv) *v = c.take<char>(lz ? 0 : (size_t)P.n * P.Lmax * vb);
@@ -537,9 +539,12 @@ static int h_dev_entry(int n, int nnz_a, const int* d_ia, const int* d_ja, const
         fp.lam = B.lam;
         fp.ne = P.ne;
         fp.active = 1;
+        fp.amax = B.lzmax;
+        if (ce == cudaSuccess) ce = cudaMemsetAsync(B.lzmax, 0, sizeof(double), s);
+        if (ce == cudaSuccess) ce = launch_krylov_scan(n, nullptr, nullptr, nullptr, 2 * (size_t)nnz_a, d_a, B.lzmax, s);
         if (ce == cudaSuccess) ce = cudaMemcpyAsync(B.lzpp, pp.data(), sizeof(int) * pp.size(), cudaMemcpyHostToDevice, s);
         if (ce == cudaSuccess) ce = cudaMemcpyAsync(B.lzprob, &fp, sizeof(fp), cudaMemcpyHostToDevice, s);
-        if (ce == cudaSuccess) ce = launch_krylov_pack_hermitian(n, d_ia, d_ja, A.v, B.lzpp, P.fp64, B.lzpk, s);
+        if (ce == cudaSuccess) ce = launch_krylov_pack_hermitian(n, d_ia, d_ja, A.v, B.lzpp, B.lzmax, P.fp64, B.lzpk, s);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);  // pp and fp are host temporaries
         if (ce != cudaSuccess) return ret(cuda_error(ce, "packed rows"));
     } else if (!P.fp64) {  // complex float copies of the values for the filter

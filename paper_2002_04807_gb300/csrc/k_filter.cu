@@ -1451,8 +1451,10 @@ __global__ void fold_dq(const FiltProb* probs, int nprob, int mt, const T* dQ, d
 // entries [pp[i], pp[i+1]) of out, its (first) diagonal entry first, then the
 // other stored entries in order; entries past the row's nonzeros are (-1, 0).
 // One warp per row.
-__global__ void pack_csr(int n, const int* ia, const int* ja, const double* av, const int* pp, int fp64, void* out)
+__global__ void pack_csr(int n, const int* ia, const int* ja, const double* av, const int* pp, int fp64, void* out,
+                         const double* amax)
 {
+    const double sc = amax ? krylov_scale(*amax) : 1.0;
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
@@ -1474,7 +1476,7 @@ __global__ void pack_csr(int n, const int* ia, const int* ja, const double* av, 
             int src = -1;
             if (q < len) src = dpos < 0 ? q : (q == 0 ? dpos : (q - 1 < dpos ? q - 1 : q));
             const int j = src >= 0 ? ja[s + src] : -1;
-            const double v = src >= 0 ? av[s + src] : 0.0;
+            const double v = src >= 0 ? av[s + src] * sc : 0.0;
             if (fp64) ((int4*)out)[t] = make_int4(j, 0, __double2loint(v), __double2hiint(v));
             else ((int2*)out)[t] = make_int2(j, __float_as_int((float)v));
         }
@@ -1503,12 +1505,12 @@ cudaError_t launch_fold_dq(const FilterArgs& a, long long max_total, bool fp64, 
 }
 
 cudaError_t launch_pack_csr(int n, const int* ia, const int* ja, const double* av, const int* pp, bool fp64, void* out,
-                            cudaStream_t s)
+                            cudaStream_t s, const double* amax)
 {
     if (n <= 0) return cudaSuccess;
     long long blocks = ((long long)n + 7) / 8;
     if (blocks > 4096) blocks = 4096;
-    pack_csr<<<(int)blocks, 256, 0, s>>>(n, ia, ja, av, pp, fp64 ? 1 : 0, out);
+    pack_csr<<<(int)blocks, 256, 0, s>>>(n, ia, ja, av, pp, fp64 ? 1 : 0, out, amax);
     count_launches(1);
     return cudaGetLastError();
 }

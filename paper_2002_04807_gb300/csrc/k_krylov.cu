@@ -37,6 +37,11 @@
 //             two CTAs per SM, all tiles at once: for problems whose ranges do
 //             not fit, or where the sums of the resident form's many narrow
 //             tiles cost more than the traffic.
+// A and the shifts are multiplied by a power of two that brings A's largest
+// entry near 1 (krylov_scale; the solutions by the same factor at the end), and
+// the pivots of z_e - T_j are carried in the filter's real type: no square
+// leaves its range for matrices of any size, and a pair of an FP64 pass stops
+// where FP64 recurrences stop it.
 // What bounds it (GB300, 2.07 GHz).  Cached, 7-point 64^3, 150 float columns:
 // 24 ms a pass of 80 steps and 222 (node, step) pairs against 154 ms with COCG
 // per node; a step moves 0.94 GB, A 130 us (3.6 TB/s: the gather's reads
@@ -122,6 +127,12 @@ template <> struct LzSum<double> {
         return o;
     }
     __device__ __forceinline__ double value() const { return h; }
+};
+
+// A (node, column) pair while it iterates: pivot of z_e - T_j, (|r| / |b|)^2.
+template <typename T>
+struct alignas(4 * sizeof(T)) LzPair {
+    T re, im, f2, pad;
 };
 
 // ---------------------------------------------------------------- packed rows
@@ -249,6 +260,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
     __shared__ S red[kLzThreads];
     __shared__ T s_al[COLS], s_inv[COLS], s_bt[COLS];
     __shared__ int s_unit;
+    __shared__ double s_zs;  // factor of A and the shifts
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int l = tid & (LPR - 1), slot = tid / LPR;
     const int nc = a.nc, team = blockIdx.x / nc, c = blockIdx.x - team * nc;
@@ -262,7 +274,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
     double* bt_g = al_g + (size_t)(a.maxit + 2) * COLS;               // beta_{j+1}, row j
     T* g_g = (T*)a.g + (size_t)team * a.maxit * COLS;
     const int npair = COLS * a.ne;
-    float4* pst = a.pair + (size_t)team * npair;  // (pivot re, im, (|r|/|b|)^2, -)
+    LzPair<T>* pst = (LzPair<T>*)a.pair + (size_t)team * npair;
     int* kst = a.kstop + (size_t)team * npair;    // step at which the pair stopped, -1 while it iterates
     double2* piv = a.piv + (size_t)team * COLS * a.nl * a.maxit;
 
@@ -308,6 +320,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
         const FiltProb& P = a.probs[un.x];
         const int n = P.n, g = un.y, m0 = P.m0;
         const int mk = P.mk ? min(*P.mk, m0) : m0;
+        if (tid == 0) s_zs = krylov_scale(*P.amax);  // read after the sums of init
         const int rpc = krylov_rpc(n, nc);
         const int r0 = RES ? min(n, c * rpc) : 0;
         const int rows = RES ? min(n, r0 + rpc) - r0 : 0;
@@ -357,7 +370,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                 bt_g[tid] = (double)b;
                 // the pairs of this column: pivot, relative residual, stop step
                 for (int e = 0; e < a.ne; ++e) {
-                    pst[e * COLS + tid] = make_float4(0.f, 0.f, 1.f, 0.f);
+                    pst[e * COLS + tid] = {T(0), T(0), T(1), T(0)};
                     kst[e * COLS + tid] = ok ? -1 : 0;
                 }
             }
@@ -601,7 +614,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                 const double b2 = red[tid].value();
                 const T b = (T)sqrt(b2);
                 const T iv = s_inv[tid];
-                const bool fine = b > T(1e-37);
+                const bool fine = b > T(sizeof(T) == 4 ? 1e-37 : 1e-300);
                 s_bt[tid] = b * iv;  // beta_{j+1} / beta_j
                 s_inv[tid] = fine ? T(1) / b : T(0);
                 if (c == 0) bt_g[(size_t)j * COLS + tid] = (double)b;
@@ -618,23 +631,22 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                 for (int pr = tid; pr < npair; pr += kLzThreads) {
                     if (kst[pr] >= 0) continue;
                     const int e = pr / COLS, cl = pr % COLS;
-                    float4 st = pst[pr];
-                    const float al = (float)s_al[cl], bn = (float)bt_g[(size_t)j * COLS + cl];
-                    const float bj = (float)bt_g[(size_t)(j - 1) * COLS + cl];
-                    float dr = (float)(P.zw[4 * e] - (double)al), di = (float)P.zw[4 * e + 1];
+                    const LzPair<T> st = pst[pr];
+                    const T bn = (T)bt_g[(size_t)j * COLS + cl], bj = (T)bt_g[(size_t)(j - 1) * COLS + cl];
+                    T dr = (T)(P.zw[4 * e] * s_zs - (double)s_al[cl]), di = (T)(P.zw[4 * e + 1] * s_zs);
                     if (j > 1) {
-                        const float w = bj * bj / (st.x * st.x + st.y * st.y);
-                        dr -= w * st.x;
-                        di += w * st.y;
+                        const T w = bj * bj / (st.re * st.re + st.im * st.im);
+                        dr -= w * st.re;
+                        di += w * st.im;
                     }
-                    const float dd = dr * dr + di * di;
-                    const float f2 = st.z * (bn * bn / dd);
-                    if (!(dd > 0.f) || !isfinite(f2)) {
+                    const T dd = dr * dr + di * di;
+                    const T f2 = st.f2 * (bn * bn / dd);
+                    if (!(dd > T(0)) || !isfinite(f2)) {
                         kst[pr] = j - 1;  // no usable step: keep the last iterate
                     } else if ((double)f2 <= a.tol2) {
                         kst[pr] = j;
                     } else {
-                        pst[pr] = make_float4(dr, di, f2, 0.f);
+                        pst[pr] = {dr, di, f2, T(0)};
                         more = 1;
                     }
                 }
@@ -678,6 +690,11 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                         cr = (wr * dr + wi * zi) / d2;
                         ci = (wi * dr - wr * zi) / d2;
                     }
+                    const double zs = s_zs;  // (z - A)^{-1} = zs (zs z - zs A)^{-1}
+                    zr *= zs;
+                    zi *= zs;
+                    cr *= zs;
+                    ci *= zs;
                 }
                 int kmax = ks;
                 for (int o = 16; o > 0; o >>= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
@@ -792,9 +809,22 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
 
 // ---------------------------------------------------------------- packed rows
 // *wide: rows that need more than eight entries (their own row's included,
-// stored or not).
-__global__ void __launch_bounds__(256) krylov_scan(int n, const int* __restrict__ ia, const int* __restrict__ ja, int* wide)
+// stored or not).  *amax: the largest |v| (the bits of doubles >= 0 are ordered
+// as they are; a NaN comes out as one).
+__global__ void __launch_bounds__(256) krylov_scan(int n, const int* __restrict__ ia, const int* __restrict__ ja, int* wide,
+                                                   size_t count, const double* __restrict__ v, unsigned long long* amax)
 {
+    unsigned long long most = 0;
+    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < count; p += (size_t)gridDim.x * blockDim.x) {
+        const unsigned long long x = (unsigned long long)__double_as_longlong(fabs(v[p]));
+        if (x > most) most = x;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, most, o);
+        if (x > most) most = x;
+    }
+    if ((threadIdx.x & 31) == 0 && most > *(volatile unsigned long long*)amax) atomicMax(amax, most);
+    if (!ja) return;
     int w = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int p0 = ia[i], len = ia[i + 1] - p0;
@@ -805,10 +835,11 @@ __global__ void __launch_bounds__(256) krylov_scan(int n, const int* __restrict_
     if (__syncthreads_or(w) && threadIdx.x == 0) *wide = 1;
 }
 
-cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, cudaStream_t s)
+cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, size_t count, const double* v, double* amax,
+                               cudaStream_t s)
 {
     const int grid = std::max(1, std::min((n + 255) / 256, num_sms() * 8));
-    krylov_scan<<<grid, 256, 0, s>>>(n, ia, ja, wide);
+    krylov_scan<<<grid, 256, 0, s>>>(n, ia, ja, wide, count, v, (unsigned long long*)amax);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -816,14 +847,17 @@ cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, c
 // Rows of at most eight entries as eight packed (position, value) entries at
 // 8 i: the own row first (value 0 when not stored), the neighbours inside the
 // row's range of rpc rows from the front, the others from the end backwards,
-// padding (position -1, value 0) between.  The last kLzFar positions are rows;
+// padding (position -1, value 0) between; values multiplied by the filter's
+// scale.  The last kLzFar positions are rows;
 // the others are rows relative to the range when all of them lie in it, else
 // (and for rpc 0) rows, and the own position is stored as ~row to say so.
 // Eight threads per row.
 template <typename E>
 __global__ void __launch_bounds__(256) krylov_pack(int n, int rpc, const int* __restrict__ ia, const int* __restrict__ ja,
-                                                   const double* __restrict__ av, E* __restrict__ out)
+                                                   const double* __restrict__ av, const double* __restrict__ amax,
+                                                   E* __restrict__ out)
 {
+    const double sc = krylov_scale(*amax);
     const int l = threadIdx.x & 7;
     const unsigned mine = 0xffu << (threadIdx.x & 24);
     for (int i0 = blockIdx.x * (blockDim.x / 8); i0 < n; i0 += gridDim.x * (blockDim.x / 8)) {
@@ -831,7 +865,7 @@ __global__ void __launch_bounds__(256) krylov_pack(int n, int rpc, const int* __
         if (i >= n) continue;  // whole groups of eight
         const int lo = rpc > 0 ? i / rpc * rpc : 0, p0 = ia[i], len = ia[i + 1] - p0;
         const int jj = l < len ? ja[p0 + l] : -1;
-        const double v = l < len ? av[p0 + l] : 0.0;
+        const double v = l < len ? av[p0 + l] * sc : 0.0;
         const unsigned has = __ballot_sync(mine, jj == i) & mine;
         const int d = has ? (__ffs(has) - 1) & 7 : -1;  // the own row's (first) entry
         const bool near = jj >= 0 && l != d && rpc > 0 && (unsigned)(jj - lo) < (unsigned)rpc;
@@ -854,12 +888,12 @@ __global__ void __launch_bounds__(256) krylov_pack(int n, int rpc, const int* __
     }
 }
 
-cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, bool fp64, void* out,
-                               cudaStream_t s)
+cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, const double* amax, bool fp64,
+                               void* out, cudaStream_t s)
 {
     const int grid = std::max(1, std::min((n + 31) / 32, num_sms() * 16));
-    if (fp64) krylov_pack<int4><<<grid, 256, 0, s>>>(n, rpc, ia, ja, av, (int4*)out);
-    else krylov_pack<int2><<<grid, 256, 0, s>>>(n, rpc, ia, ja, av, (int2*)out);
+    if (fp64) krylov_pack<int4><<<grid, 256, 0, s>>>(n, rpc, ia, ja, av, amax, (int4*)out);
+    else krylov_pack<int2><<<grid, 256, 0, s>>>(n, rpc, ia, ja, av, amax, (int2*)out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -872,8 +906,9 @@ cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, con
 template <typename E, typename V2>
 __global__ void __launch_bounds__(256) krylov_pack_hermitian(int n, const int* __restrict__ ia, const int* __restrict__ ja,
                                                              const V2* __restrict__ av, const int* __restrict__ pp,
-                                                             E* __restrict__ out)
+                                                             const double* __restrict__ amax, E* __restrict__ out)
 {
+    const double sc = krylov_scale(*amax);
     const int lane = threadIdx.x & 31, nw = (gridDim.x * blockDim.x) >> 5;
     for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
         const int p0 = ia[i], len = ia[i + 1] - p0;
@@ -887,7 +922,7 @@ __global__ void __launch_bounds__(256) krylov_pack_hermitian(int n, const int* _
                 if (q < len) {
                     j = 2 * ja[p0 + q] + im;
                     const V2 a = av[p0 + q];
-                    v = im == h ? (double)a.x : (h ? (double)a.y : -(double)a.y);
+                    v = sc * (im == h ? (double)a.x : (h ? (double)a.y : -(double)a.y));
                 }
                 if constexpr (sizeof(E) == 8) out[t] = make_int2(j, __float_as_int((float)v));
                 else out[t] = make_int4(j, 0, __double2loint(v), __double2hiint(v));
@@ -896,12 +931,12 @@ __global__ void __launch_bounds__(256) krylov_pack_hermitian(int n, const int* _
     }
 }
 
-cudaError_t launch_krylov_pack_hermitian(int n, const int* ia, const int* ja, const double2* av, const int* pp, bool fp64,
-                                         void* out, cudaStream_t s)
+cudaError_t launch_krylov_pack_hermitian(int n, const int* ia, const int* ja, const double2* av, const int* pp,
+                                         const double* amax, bool fp64, void* out, cudaStream_t s)
 {
     const int grid = std::max(1, std::min((n + 7) / 8, num_sms() * 16));
-    if (fp64) krylov_pack_hermitian<int4><<<grid, 256, 0, s>>>(n, ia, ja, av, pp, (int4*)out);
-    else krylov_pack_hermitian<int2><<<grid, 256, 0, s>>>(n, ia, ja, av, pp, (int2*)out);
+    if (fp64) krylov_pack_hermitian<int4><<<grid, 256, 0, s>>>(n, ia, ja, av, pp, amax, (int4*)out);
+    else krylov_pack_hermitian<int2><<<grid, 256, 0, s>>>(n, ia, ja, av, pp, amax, (int2*)out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -933,7 +968,7 @@ static double krylov_size(KrylovPlan& k, bool fp64, int lanes, int n, int ne, in
     k.ne = ne;
     k.slot_vecs = (size_t)n * lanes;
     k.team_bytes = ((size_t)maxit + 1) * k.slot_vecs * 16;
-    return (double)k.team_bytes + (double)k.cols * k.nl * 16.0 * maxit + (double)k.cols * (24.0 * maxit + 20.0 * ne);
+    return (double)k.team_bytes + (double)k.cols * k.nl * 16.0 * maxit + (double)k.cols * (24.0 * maxit + 36.0 * ne);
 }
 
 KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes)
@@ -1013,7 +1048,7 @@ size_t krylov_layout(const KrylovPlan& k, char* base, KrylovArgs& a)
     a.part = take(nt * 2 * k.nc * k.cols * 8);
     a.coef = (double*)take(nt * 2 * (mi + 2) * k.cols * sizeof(double));
     a.g = take(nt * mi * k.lanes * 16);
-    a.pair = (float4*)take(nt * k.cols * k.ne * sizeof(float4));
+    a.pair = take(nt * k.cols * k.ne * sizeof(LzPair<double>));
     a.kstop = (int*)take(nt * k.cols * k.ne * sizeof(int));
     a.piv = (double2*)take(nt * k.cols * k.nl * mi * sizeof(double2));
     a.bar = (unsigned*)take((nt + 1) * 128);  // team counters, then the unit queue
