@@ -263,6 +263,11 @@ int feast_scsr_solve_batched(int np, const feast_problem* probs, int* fpm, feast
  * the vectors of one COCG per node is used for that, several times slower. */
 size_t feast_scsr_workspace_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm);
 
+/* The least workspace, in bytes, that the same calls accept: for a problem
+ * without B that of one COCG per node, where it is smaller than the size above;
+ * with a B the size above. */
+size_t feast_scsr_workspace_min_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm);
+
 /* Same as feast_scsr_solve with the matrices and X already on the device.
  * d_ia/d_ja/d_a: 0-based CSR of A in full storage (device); d_ib/d_jb/d_b the
  * same for B or NULL for B = I; d_x: device, column-major n x m0, in/out as x

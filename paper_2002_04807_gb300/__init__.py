@@ -40,6 +40,7 @@ from ._lib import (  # noqa: F401
     feast_scsr_extreme_dev,
     feast_scsr_grad,
     feast_scsr_workspace_bytes,
+    feast_scsr_workspace_min_bytes,
     feast_set_wait_limit,
     feast_shifted_spmm_dev,
     feast_sym_eig_dev,

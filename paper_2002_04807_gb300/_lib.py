@@ -26,6 +26,7 @@ _SIGS = {
     "feast_scsr_solve": (_i, [C.c_char, _i, _p, _p, _p, _p, _p, _p, _p, _d, _d, _p, _p, _p, _p, _p, _p, _p,
                               _p]),
     "feast_scsr_workspace_bytes": (C.c_size_t, [_i, _i, _i, _i, _p]),
+    "feast_scsr_workspace_min_bytes": (C.c_size_t, [_i, _i, _i, _i, _p]),
     "feast_scsr_solve_dev": (_i, [_i, _i, _p, _p, _p, _i, _p, _p, _p, _p, _d, _d, _p, _p, _p, _p, _p, _p, _p,
                                   _p, _p, C.c_size_t, _p]),
     "feast_filter_layout": (_i, [_i, _i, _p, _p, _p]),
@@ -250,12 +251,32 @@ def feast_scsr_workspace_bytes(n: int, nnz_a: int, nnz_b: int, m0: int, fpm) -> 
     return int(library().feast_scsr_workspace_bytes(n, nnz_a, nnz_b, m0, _ptr(f)))
 
 
+def feast_scsr_workspace_min_bytes(n: int, nnz_a: int, nnz_b: int, m0: int, fpm) -> int:
+    """The least workspace that the device drivers accept (without Krylov bases
+    for a problem with B = I: one COCG per node, several times slower)."""
+    return int(library().feast_scsr_workspace_min_bytes(n, nnz_a, nnz_b, m0, _ptr(_fpm(fpm))))
+
+
+def _workspace(n, nnz_a, nnz_b, m0, f, work, device):
+    """The caller's workspace if a call accepts its size, else a new one: of the
+    full size, or of the least one where the memory does not hold that."""
+    import torch
+
+    if work is not None and work.numel() >= feast_scsr_workspace_min_bytes(n, nnz_a, nnz_b, m0, f):
+        return work
+    try:
+        return torch.empty(feast_scsr_workspace_bytes(n, nnz_a, nnz_b, m0, f), dtype=torch.uint8, device=device)
+    except torch.cuda.OutOfMemoryError:
+        return torch.empty(feast_scsr_workspace_min_bytes(n, nnz_a, nnz_b, m0, f), dtype=torch.uint8, device=device)
+
+
 def feast_scsr_solve_dev(n: int, ia, ja, a, ib=None, jb=None, b=None, fpm=None, emin=0.0, emax=1.0,
                          m0: int = 1, x=None, work=None, stream=None) -> FeastResult:
     """Device driver: 0-based CSR as torch CUDA tensors (int32 / float64), x a
     CUDA float64 tensor holding the column-major n x m0 block (in/out; shape
     (m0, n) row-major is the same memory).  work: optional preallocated uint8
-    CUDA tensor."""
+    CUDA tensor, used when it has at least feast_scsr_workspace_min_bytes(...)
+    bytes (fewer than feast_scsr_workspace_bytes(...): without Krylov bases)."""
     import torch
 
     f = _fpm(fpm)
@@ -267,9 +288,7 @@ def feast_scsr_solve_dev(n: int, ia, ja, a, ib=None, jb=None, b=None, fpm=None, 
     if x is None:
         x = torch.zeros((m0, n), dtype=torch.float64, device=a.device)
     x = _dev(x, torch.float64)
-    need = feast_scsr_workspace_bytes(n, a.numel(), nnzb, m0, f)
-    if work is None or work.numel() < need:
-        work = torch.empty(need, dtype=torch.uint8, device=a.device)
+    work = _workspace(n, a.numel(), nnzb, m0, f, work, a.device)
     E = np.zeros(m0)
     res = np.zeros(m0)
     M, loop, info, mm = _i(0), _i(0), _i(0), _i(m0)
@@ -334,9 +353,7 @@ def feast_scsr_solve_dev_x(n: int, ia, ja, a, zne, wne, ib=None, jb=None, b=None
     if x is None:
         x = torch.zeros((m0, n), dtype=torch.float64, device=a.device)
     x = _dev(x, torch.float64)
-    need = feast_scsr_workspace_bytes(n, a.numel(), nnzb, m0, f)
-    if work is None or work.numel() < need:
-        work = torch.empty(need, dtype=torch.uint8, device=a.device)
+    work = _workspace(n, a.numel(), nnzb, m0, f, work, a.device)
     z, w = _nodes(zne, wne)
     E = np.zeros(m0)
     res = np.zeros(m0)
@@ -395,9 +412,7 @@ def feast_scsr_extreme_dev(n: int, ia, ja, a, ib=None, jb=None, b=None, fpm=None
     if x is None:
         x = torch.zeros((m0, n), dtype=torch.float64, device=a.device)
     x = _dev(x, torch.float64)
-    need = feast_scsr_workspace_bytes(n, a.numel(), nnzb, m0, f)
-    if work is None or work.numel() < need:
-        work = torch.empty(need, dtype=torch.uint8, device=a.device)
+    work = _workspace(n, a.numel(), nnzb, m0, f, work, a.device)
     E = np.zeros(m0)
     res = np.zeros(m0)
     M, loop, info, mm = _i(0), _i(0), _i(0), _i(m0)

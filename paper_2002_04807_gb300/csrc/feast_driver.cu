@@ -1313,6 +1313,12 @@ extern "C" size_t feast_scsr_workspace_bytes(int n, int nnz_a, int nnz_b, int m0
     return scsr_bytes(n, nnz_a, nnz_b, m0, fpm, true);
 }
 
+extern "C" size_t feast_scsr_workspace_min_bytes(int n, int nnz_a, int nnz_b, int m0, const int* fpm)
+{
+    if (n <= 0 || m0 <= 0 || !fpm) return 0;
+    return std::min(scsr_bytes(n, nnz_a, nnz_b, m0, fpm, true), scsr_bytes(n, nnz_a, nnz_b, m0, fpm, false));
+}
+
 // Smallest and largest Gershgorin bound over the rows (scaled by diag(scale)
 // when given).  Synchronises the stream.
 static int gersh_bounds(const int* ia, const int* ja, const double* v, int n, const double* scale, double* part,
