@@ -2411,7 +2411,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         }
         if (!fits) kinds.clear();
     }
-    const bool lz = !kinds.empty();
+    bool lz = !kinds.empty();
     long long max_units = 0;
     for (const Kind& kd : kinds) {
         long long u = 0;
@@ -2434,11 +2434,12 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         items_a_max += (long long)G[p] * ((probs[p].n + rb_min - 1) / rb_min);
         items_b += (long long)G[p] * fpv[p].nrb_b;
     }
-    // ---- device memory: one allocation carved in place
+    // ---- device memory: one allocation carved in place; without Krylov bases (COCG
+    // per node) where the device does not hold them
     DevMem dm;
     Bump bump;
     char* base = nullptr;
-    for (int pass = 0; pass < 2; ++pass) {
+    for (int pass = 0; pass < 2;) {
         bump.base = base;
         bump.off = 0;
         (void)bump.take<int>(ppA);
@@ -2484,8 +2485,17 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         (void)bump.take<double>(np);
         if (pass == 0) {
             cudaError_t e = dm.alloc(&base, bump.off + 4096);
+            if (e == cudaErrorMemoryAllocation && lz) {
+                cudaGetLastError();
+                kinds.clear();
+                lz = false;
+                lz_bytes = 0;
+                max_units = 0;
+                continue;
+            }
             if (e != cudaSuccess) return cuda_fail(e, "batched workspace");
         }
+        ++pass;
     }
     bump.base = base;
     bump.off = 0;

@@ -69,3 +69,26 @@ def test_a_device_without_room_for_the_bases(pkg, entry):
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert without and len(e) == len(ref) and np.abs(e - ref).max() <= 1e-9
+
+
+def test_batch_on_a_device_without_room_for_the_bases(pkg):
+    """Most of the device is held by tensors: the 7 GB of Krylov bases of this
+    batch do not fit, the 0.2 GB of its COCG do."""
+    f = pkg.feast_init()
+    f[1], f[2], f[3], f[17], f[41], f[44], f[45] = 8, 10, 40, 100, 1, 2, 4000
+    probs = [fw.laplace3d_potential(side=16, count=16, m0=24, seed=s) for s in range(6)]
+    batch = [dict(n=p.n, a=p.A.data, ia=p.A.indptr, ja=p.A.indices, emin=p.emin, emax=p.emax, m0=24) for p in probs]
+    st, ref = pkg.feast_scsr_solve_batched(batch, f.copy())
+    assert st == 0
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - (3 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        st, got = pkg.feast_scsr_solve_batched(batch, f.copy())
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert st == 0
+    for r, r0 in zip(got, ref):
+        assert r.info == r0.info == 0 and r.M == r0.M > 0
+        assert np.abs(r.E[: r.M] - r0.E[: r0.M]).max() <= 1e-9
