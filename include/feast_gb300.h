@@ -128,7 +128,8 @@ int feast_contour_nodes_rule(int rule, int ne, double emin, double emax, int rat
  * reduced eigensolver, [8] ms forming Ritz vectors and residuals, [9] tile
  * width W, [10] columns per group mt, [11] n, [12] bytes per complex value,
  * [13] column groups, [14] refinement loops, [15] kernel launches issued,
- * [16] rows per step-A work item, [17] 0 when step A gathers through the
+ * [16] rows per step-A work item (B = I: rows that a warp takes at once when
+ * [17] is 1, rows of a block dealt to a CTA when it is 0), [17] 0 when step A gathers through the
  * caches, 1 when it stages the rows it gathers in shared memory (windows of r
  * copied by the bulk-copy engine; B = I: each CTA keeps its rows of the
  * vectors there), 2 for the staged form with a producer warp

@@ -977,7 +977,7 @@ int setup_krylov(const Plan& P, Bufs& B, const Csr& A, cudaStream_t s)
     B.lzp = wide || P.lzr.teams == 0 || P.lzc.cost < P.lzr.cost ? &P.lzc : &P.lzr;
     krylov_layout(*B.lzp, B.lzmem, B.lz);
     B.lz.one_chunk = wide ? 0 : 1;
-    B.RB = B.lzp->resident ? 64 : 256;
+    B.RB = krylov_item_rows(*B.lzp);
     if (!wide) {
         CK(launch_krylov_pack(A.n, B.lzp->rpc, A.ia, A.ja, A.v, B.lzmax, P.fp64, B.apk, s));
         return 0;

@@ -209,6 +209,9 @@ constexpr double kKrylovBytes = 64e9;
 KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes);
 KrylovPlan krylov_plan_set(bool fp64, int np, const int* n, const int* m, int ne, int maxit, double max_bytes);
 int krylov_rows(int n, int nc);  // rows per CTA of the resident form
+// Rows of a work item of the gathered product, as feast_last_profile reports it:
+// those a warp takes at once (resident), a block dealt to a CTA (cached).
+int krylov_item_rows(const KrylovPlan& k);
 // Power of two by which the Krylov filter multiplies A and the shifts, so that
 // the steps run on entries near 1 whatever the size of A's (amax: the largest).
 __host__ __device__ inline double krylov_scale(double amax)

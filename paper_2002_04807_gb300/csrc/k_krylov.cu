@@ -944,6 +944,8 @@ cudaError_t launch_krylov_pack_hermitian(int n, const int* ia, const int* ja, co
 // ---------------------------------------------------------------- plan and launch
 int krylov_rows(int n, int nc) { return krylov_rpc(n, nc); }
 
+int krylov_item_rows(const KrylovPlan& k) { return k.resident ? 32 / k.lanes : kLzBlock; }
+
 // Bytes of Krylov bases beyond which a pass takes its tiles one team at a time.
 static constexpr double kKrylovMany = 16e9;
 
