@@ -412,8 +412,8 @@ int feast_gram_noalloc_dev(int n, int m, const double* X, const double* Y, doubl
  * column scale; products accumulated exactly in FP32 for 128 rows at a time,
  * then in 64-bit integers), the arithmetic of the solvers' projections A_Q = Q^T A Q,
  * B_Q = Q^T B Q when fpm(54) = 0 (Sec. 1.1's reduced problem, FP64 accuracy:
- * the truncation error of an element is below 2^-55 max|X[:,a]| max|Y[:,b]|
- * per row).  Device row-major n x m X, Y; C m x m.  Returns 0, -101 n <= 0,
+ * the error of an element is below 5 * 2^-53 max|X[:,a]| max|Y[:,b]| per row,
+ * beside the rounding of its sum).  Device row-major n x m X, Y; C m x m.  Returns 0, -101 n <= 0,
  * -102 m <= 0, -4 on a CUDA error. */
 int feast_gram_oz_dev(int n, int m, const double* X, const double* Y, double* C, void* stream);
 
@@ -423,7 +423,7 @@ int feast_gemm_dev(int n, int m, int k, const double* A, const double* V, double
 /* C = A V as feast_gemm_dev, from exact BF16 slice products on the tensor
  * cores under a power-of-two scale per row of A and per column of V (the
  * arithmetic of the Ritz vectors X = Q V when fpm(54) = 0; FP64 accuracy:
- * truncation below 2^-55 max|A[i,:]| max|V[:,c]| per term).  Same arguments
+ * error below 5 * 2^-53 max|A[i,:]| max|V[:,c]| per term).  Same arguments
  * and return codes as feast_gemm_dev. */
 int feast_gemm_oz_dev(int n, int m, int k, const double* A, const double* V, double* C, void* stream);
 

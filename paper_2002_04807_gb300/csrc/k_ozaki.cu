@@ -12,16 +12,17 @@
 //     x 2^-E = sum_s d_s 2^(1 - 8 s) + r, d_s in [-128, 128], |r| <= 2^-56; the
 //     digits are the bytes of F plus a bias and are exact in BF16;
 //   * X[i][a] Y[i][b] = 2^(E_a + F_b) sum_{s,t} d_s(i,a) e_t(i,b) 2^(2 - 8 (s+t)),
-//     the pairs with s + t <= kSlices + 1 are kept (28; the rest weigh below
-//     2^(-53) relative to 2^(E_a + F_b) even with every digit at its largest);
+//     the pairs with s + t <= kSlices + 1 are kept (28; the rest, six of 2^14
+//     2^-70 and smaller ones, weigh at most 6.03 2^-56 relative to 2^(E_a + F_b));
 //   * a level L = s + t has at most kSlices pairs of products of at most 2^14,
 //     so its sum over 128 rows stays below 2^24 and mma.sync accumulates it in
 //     FP32 without any rounding; every 128 rows the level sums are folded,
 //     exactly, into two 64-bit integer accumulators (oz_fold), and at the end
 //     they are turned into FP64 once and the column scales 2^(E_a + F_b) are
 //     applied.
-// With kSlices = 7 the kept part is exact and the truncation error of an
-// element is below 2^-55 |2^E_a| |2^F_b| per row: at FP64 level.
+// With kSlices = 7 the kept part is exact and the error of an element is below
+// 9 2^-56 2^(E_a + F_b) per row (the pairs left out and r of both factors; a
+// power of two is at most twice its column's largest value): at FP64 level.
 // Eight 7-bit digits of |x| (36 pairs) gave the same error; cutting them took
 // 60 integer instructions a value and the ALU was the busiest unit (60 %, tensor
 // pipe 34 %: 1.31 ms at n = 262,144, m = 150).  A byte becomes a digit by one
