@@ -221,9 +221,10 @@ __host__ __device__ inline double krylov_scale(double amax)
     return ldexp(1.0, e < -1000 ? 1000 : -e);
 }
 size_t krylov_layout(const KrylovPlan& k, char* base, KrylovArgs& a);
-// amax (zeroed): the largest |v| of count values; wide (zeroed), unless ja is
-// null: set when a row needs more than eight packed entries.
-cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, size_t count, const double* v, double* amax,
+// amax (zeroed): the largest |v| of the matrix's entries (parts = 2: of their real
+// and imaginary parts); wide (zeroed), unless ja is null: set when a row needs
+// more than eight packed entries.
+cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, int parts, const double* v, double* amax,
                                cudaStream_t s);
 cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, const double* amax, bool fp64,
                                void* out, cudaStream_t s);

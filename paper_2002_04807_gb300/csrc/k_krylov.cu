@@ -812,10 +812,12 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
 // stored or not).  *amax: the largest |v| (the bits of doubles >= 0 are ordered
 // as they are; a NaN comes out as one).
 __global__ void __launch_bounds__(256) krylov_scan(int n, const int* __restrict__ ia, const int* __restrict__ ja, int* wide,
-                                                   size_t count, const double* __restrict__ v, unsigned long long* amax)
+                                                   int parts, const double* __restrict__ v, unsigned long long* amax)
 {
     unsigned long long most = 0;
-    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < count; p += (size_t)gridDim.x * blockDim.x) {
+    const size_t end = (size_t)ia[n] * parts;  // not all that the arrays may hold
+    for (size_t p = (size_t)ia[0] * parts + blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < end;
+         p += (size_t)gridDim.x * blockDim.x) {
         const unsigned long long x = (unsigned long long)__double_as_longlong(fabs(v[p]));
         if (x > most) most = x;
     }
@@ -835,11 +837,11 @@ __global__ void __launch_bounds__(256) krylov_scan(int n, const int* __restrict_
     if (__syncthreads_or(w) && threadIdx.x == 0) *wide = 1;
 }
 
-cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, size_t count, const double* v, double* amax,
+cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, int parts, const double* v, double* amax,
                                cudaStream_t s)
 {
     const int grid = std::max(1, std::min((n + 255) / 256, num_sms() * 8));
-    krylov_scan<<<grid, 256, 0, s>>>(n, ia, ja, wide, count, v, (unsigned long long*)amax);
+    krylov_scan<<<grid, 256, 0, s>>>(n, ia, ja, wide, parts, v, (unsigned long long*)amax);
     count_launches(1);
     return cudaGetLastError();
 }

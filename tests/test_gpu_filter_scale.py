@@ -58,6 +58,17 @@ def test_filter_is_independent_of_units(pkg, kind, mixed, rii, power):
     assert np.array_equal(Q, ref)
 
 
+def test_values_beyond_the_rows_are_not_read(pkg):
+    """Arrays longer than ia[n], as a caller with room to spare passes them."""
+    A = _grid((40,), 9)
+    Y = fw.gaussian_block(A.n, 4, 10)
+    ref, _ = _filter(pkg, A, Y, 1, 0.0, 1.0)
+    A.indices = np.concatenate([A.indices, np.zeros(9, dtype=A.indices.dtype)])
+    A.data = np.concatenate([A.data, np.full(9, 1e300)])
+    Q, _ = _filter(pkg, A, Y, 1, 0.0, 1.0)
+    assert np.array_equal(Q, ref)
+
+
 def test_filter_of_a_shifted_spectrum_stops_alike(pkg):
     """A + s I with a shift of 2^26 on a spectrum of width 4 (both exact): the
     nodes are rounded to 7.5e-9, a quarter of a millionth of their distance (0.03)
