@@ -2244,6 +2244,11 @@ struct Bump {
     }
 };
 
+// Packed entries of an n-row matrix: rows padded to eights, a row at least one
+// chunk.  Whole chunks, because the problems of a batch follow each other and a
+// chunk is read 16 bytes at a time (two single-precision entries).
+long long packed_entries(size_t nnz, int n) { return (std::max((long long)nnz + 7LL * n, 8LL * n) + 7) / 8 * 8; }
+
 // rows-per-item choices tried by the autotuner, and the cache of its picks
 // keyed by (total rows / 2^16, tile width, precision)
 std::vector<std::pair<long long, int>> g_rb_cache;
@@ -2365,10 +2370,10 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         nnzA += (long long)aja[p].size();
         nnzB += (long long)bja[p].size();
         ppA += n + 1;
-        pkA += std::max((long long)aja[p].size() + 7LL * n, 8LL * n);
+        pkA += packed_entries(aja[p].size(), n);
         if (bmode == 2) {
             ppB += n + 1;
-            pkB += (long long)bja[p].size() + 7LL * n;
+            pkB += packed_entries(bja[p].size(), n);
         }
         maxm = std::max(maxm, m);
     }
@@ -2610,7 +2615,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
                     f.bpp = d_bpp + oppb;
                     f.bpk = d_bpk + opkb * pkz;
                     oppb += n + 1;
-                    opkb += (long long)bja[p].size() + 7LL * n;
+                    opkb += packed_entries(bja[p].size(), n);
                 }
                 ob += n + 1;
                 onzb += (long long)bja[p].size();
@@ -2618,7 +2623,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
             oa += n + 1;
             onz += (long long)aja[p].size();
             opp += n + 1;
-            opk += std::max((long long)aja[p].size() + 7LL * n, 8LL * n);
+            opk += packed_entries(aja[p].size(), n);
             std::vector<double> zw;
             contour(fpm[15], ne, probs[p].emin, probs[p].emax, fpm[17] / 100.0, zw);
             std::copy(zw.begin(), zw.end(), zw_all.begin() + (size_t)p * ne * 4);
