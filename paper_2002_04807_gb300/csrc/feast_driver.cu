@@ -2377,42 +2377,54 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
         }
         maxm = std::max(maxm, m);
     }
-    // B = I: one Krylov space per column (k_krylov.cu), when every row packs into
-    // eight entries; problems of similar size share a launch (kinds), the
-    // largest first
+    // B = I: one Krylov space per column (k_krylov.cu).  Problems of similar size
+    // share a launch (kinds), the largest first; those with a row of more than
+    // eight entries have kinds of their own, in the cached form, so that they do
+    // not decide for the others
     struct Kind {
         KrylovPlan plan;
         KrylovArgs args = {};
+        bool one_chunk = true;  // every row packs into eight entries
         std::vector<int> probs;
     };
     std::vector<Kind> kinds;
     size_t lz_bytes = 0;
     if (!hasB && fpm[50] == 0) {
-        bool fits = true;
-        for (int p = 0; p < np && fits; ++p)
-            for (int i = 0; i < probs[p].n && fits; ++i) {
+        std::vector<int> order[2];  // problems of short rows, of long ones
+        for (int p = 0; p < np; ++p) {
+            bool small = true;
+            for (int i = 0; i < probs[p].n && small; ++i) {
                 const int len = aia[p][i + 1] - aia[p][i];
                 const int* c = aja[p].data() + aia[p][i];
-                fits = len < 8 || (len == 8 && std::find(c, c + len, i) != c + len);
+                small = len < 8 || (len == 8 && std::find(c, c + len, i) != c + len);
             }
-        std::vector<int> order(np);
-        for (int p = 0; p < np; ++p) order[p] = p;
-        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return probs[x].n > probs[y].n; });
-        for (int q = 0; q < np && fits;) {
-            // from the largest problem left, those of more than half its rows (all
-            // the rest once one CTA holds a four-column tile)
-            const int top = probs[order[q]].n, least = top > 6912 ? top / 2 : 0;
-            Kind kd;
-            std::vector<int> kn, km;
-            for (; q < np && probs[order[q]].n > least; ++q) {
-                kd.probs.push_back(order[q]);
-                kn.push_back(probs[order[q]].n);
-                km.push_back(probs[order[q]].m0);
+            order[small ? 0 : 1].push_back(p);
+        }
+        bool fits = true;
+        for (int w = 0; w < 2; ++w) {
+            const std::vector<int>& ord = order[w];
+            std::stable_sort(order[w].begin(), order[w].end(), [&](int x, int y) { return probs[x].n > probs[y].n; });
+            for (size_t q = 0; q < ord.size() && fits;) {
+                // from the largest problem left, those of more than half its rows (all
+                // the rest once one CTA holds a four-column tile)
+                const int top = probs[ord[q]].n, least = top > 6912 ? top / 2 : 0;
+                Kind kd;
+                kd.one_chunk = w == 0;
+                std::vector<int> kn, km;
+                for (; q < ord.size() && probs[ord[q]].n > least; ++q) {
+                    kd.probs.push_back(ord[q]);
+                    kn.push_back(probs[ord[q]].n);
+                    km.push_back(probs[ord[q]].m0);
+                }
+                auto plan = [&](bool resident) {
+                    return krylov_plan_set(fp64, resident, (int)kn.size(), kn.data(), km.data(), ne, maxit, kKrylovBatchBytes);
+                };
+                if (kd.one_chunk) kd.plan = plan(true);
+                if (kd.plan.teams == 0) kd.plan = plan(false);
+                fits = kd.plan.teams > 0;
+                if (fits) lz_bytes = std::max(lz_bytes, krylov_layout(kd.plan, nullptr, kd.args));
+                kinds.push_back(std::move(kd));
             }
-            kd.plan = krylov_plan_set(fp64, (int)kn.size(), kn.data(), km.data(), ne, maxit, kKrylovBatchBytes);
-            fits = kd.plan.teams > 0;
-            if (fits) lz_bytes = std::max(lz_bytes, krylov_layout(kd.plan, nullptr, kd.args));
-            kinds.push_back(std::move(kd));
         }
         if (!fits) kinds.clear();
     }
@@ -2552,10 +2564,11 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
     int2* d_units = bump.take<int2>(max_units);
     char* d_jwork = bump.take<char>(jacobi_batch_bytes(np));
     double* d_amax = bump.take<double>(np);  // largest |entry| of every A
-    std::vector<int> rpc(np, 0);  // rows per CTA of each problem's resident form
+    std::vector<int> rpc(np, -1);  // rows per CTA of the resident form, 0: cached; -1: packed in chunks
     for (Kind& kd : kinds) {
         krylov_layout(kd.plan, d_lz, kd.args);
-        for (const int p : kd.probs) rpc[p] = krylov_rows(probs[p].n, kd.plan.nc);
+        for (const int p : kd.probs)
+            if (kd.one_chunk) rpc[p] = kd.plan.resident ? krylov_rows(probs[p].n, kd.plan.nc) : 0;
     }
     cudaStream_t s = nullptr;
     CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
@@ -2584,7 +2597,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
             f.ia = b.ia = d_ia + oa;
             f.ja = b.ja = d_ja + onz;
             f.av = b.av = d_a + onz;
-            if (lz) {
+            if (rpc[p] >= 0) {
                 CK(launch_krylov_pack(n, rpc[p], d_ia + oa, d_ja + onz, d_a + onz, d_amax + p, fp64, d_apk + opk * pkz, s));
             } else {
                 // padded chunk pointers from the host copy
@@ -2592,7 +2605,8 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
                 for (int i = 0; i < n; ++i) pp[i + 1] = pp[i] + (aia[p][i + 1] - aia[p][i] + 7) / 8 * 8;
                 CK(cudaMemcpyAsync(d_app + opp, pp.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s));
                 CK(cudaStreamSynchronize(s));
-                CK(launch_pack_csr(n, d_ia + oa, d_ja + onz, d_a + onz, d_app + opp, fp64, d_apk + opk * pkz, s));
+                CK(launch_pack_csr(n, d_ia + oa, d_ja + onz, d_a + onz, d_app + opp, fp64, d_apk + opk * pkz, s,
+                                   lz ? d_amax + p : nullptr));
             }
             f.app = d_app + opp;
             f.apk = d_apk + opk * pkz;
@@ -2831,7 +2845,7 @@ extern "C" int feast_scsr_solve_batched(int np, const feast_problem* probs, int*
             a.nbp = nbp;
             a.nbatch = nbatch;
             a.rii = 1;
-            a.one_chunk = 1;
+            a.one_chunk = kd.one_chunk ? 1 : 0;
             a.tol2 = tol * tol;
             a.err = d_k;
             a.limit = wait_limit_cycles();

@@ -207,7 +207,7 @@ struct KrylovArgs {
 // Device memory a contour pass of one problem may take for its Krylov bases.
 constexpr double kKrylovBytes = 64e9;
 KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes);
-KrylovPlan krylov_plan_set(bool fp64, int np, const int* n, const int* m, int ne, int maxit, double max_bytes);
+KrylovPlan krylov_plan_set(bool fp64, bool resident, int np, const int* n, const int* m, int ne, int maxit, double max_bytes);
 int krylov_rows(int n, int nc);  // rows per CTA of the resident form
 // Rows of a work item of the gathered product, as feast_last_profile reports it:
 // those a warp takes at once (resident), a block dealt to a CTA (cached).

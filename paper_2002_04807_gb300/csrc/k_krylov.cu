@@ -1000,24 +1000,24 @@ KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit
     return best;
 }
 
-// Plan of the resident form for a set of problems (np of them, n[i] rows and
-// m[i] columns) whose tiles the teams take from one queue; teams = 0 when the
-// largest does not fit.
-KrylovPlan krylov_plan_set(bool fp64, int np, const int* n, const int* m, int ne, int maxit, double max_bytes)
+// Plan for a set of problems (np of them, n[i] rows and m[i] columns) whose
+// tiles the teams take from one queue; teams = 0 when the largest does not fit.
+KrylovPlan krylov_plan_set(bool fp64, bool resident, int np, const int* n, const int* m, int ne, int maxit, double max_bytes)
 {
     KrylovPlan best;
-    const int sms = num_sms(), maxn = *std::max_element(n, n + np);
+    const int ctas = resident ? num_sms() : 2 * num_sms(), maxn = *std::max_element(n, n + np);
     for (int lanes = kLzMaxLanes; lanes >= 1; lanes /= 2) {
+        if (!resident && lanes != kLzMaxLanes) break;
         KrylovPlan k;
-        k.resident = true;
+        k.resident = resident;
         const double per_team = krylov_size(k, fp64, lanes, maxn, ne, maxit);
         if (per_team > max_bytes) continue;
         long long units = 0;
         for (int i = 0; i < np; ++i) units += (m[i] + k.cols - 1) / k.cols;
-        for (k.nc = 1; k.nc <= sms; k.nc *= 2) {
-            k.rpc = krylov_rpc(maxn, k.nc);
+        for (k.nc = 1; k.nc <= ctas; k.nc *= 2) {
+            k.rpc = resident ? krylov_rpc(maxn, k.nc) : 0;
             if ((size_t)k.rpc * lanes * 32 > kLzSmem) continue;
-            k.teams = (int)std::min<double>({(double)(sms / k.nc), (double)units, std::max(1.0, max_bytes / per_team)});
+            k.teams = (int)std::min<double>({(double)(ctas / k.nc), (double)units, std::max(1.0, max_bytes / per_team)});
             double sum = 0.0, longest = 0.0;
             for (int i = 0; i < np; ++i) {
                 const double us = krylov_tile_cost(k, fp64, n[i]);
