@@ -72,9 +72,10 @@ def config_dict(p, extra=None):
     d = {"workload": f"laplace3d_7pt_{round(p.n ** (1 / 3))}^3_potential_U[0,0.5]_seed1",
          "N": p.n, "nnz": p.A.nnz, "M0": p.m0, "Ne": p.ne, "contour_ratio_pct": p.ratio,
          "interval": [p.emin, round(p.emax, 6)], "B": "identity", "tol": RES_TOL,
-         "inner_solver": f"COCG, fpm(45)={INNER[0]} (1e-{INNER[0]}), fpm(46)={INNER[1]}, one node per batch "
-                         "(fpm(50)=1)",
-         "l2": "inputs larger than L2 (each filter block vector 2.5 GB)"}
+         "inner_solver": ("COCG, one node per batch" if ROWS_PER_ITEM else
+                          "COCG's iterates at all nodes from one Krylov space per column")
+                         + f", fpm(45)={INNER[0]} (1e-{INNER[0]}), fpm(46)={INNER[1]}",
+         "l2": f"inputs larger than L2 (each of a pass's basis blocks {p.n * p.m0 * 4 / 1e6:.0f} MB)"}
     if extra:
         d.update(extra)
     return d
@@ -460,7 +461,7 @@ def run_reference(args):
            "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * wall / args.steps,
            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
            "data": "synthetic (seeded generator, no dataset)", "impl": "reference",
-           "config": config_dict(p, {"precision": "FP64 oracle", "M": Mo, "filter_passes": passes}),
+           "config": config_dict(p, {"precision": "FP64 oracle", "inner_solver": "COCG to 1e-13", "M": Mo, "filter_passes": passes}),
            "cpu_baseline": {"value": value, "unit": UNIT, "cores": cores, "kind": "oracle", "sample": samples},
            "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
     print(json.dumps(out))

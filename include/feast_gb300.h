@@ -246,8 +246,9 @@ typedef struct feast_result {
 /* Many independent problems of uneven size and interval solved together (the
  * guide's first level of parallelism, Sec. 1.1: separate search intervals).
  * One set of filter launches serves all unfinished problems; the COCG steps
- * replay as a captured CUDA graph (problems with B; without, a pass is one
- * launch per class of sizes); the
+ * replay as a captured CUDA graph (problems with B, and batches whose Krylov
+ * bases the device does not hold; without B, a pass is one launch per class of
+ * sizes and row lengths); the
  * rows per work item of the gathering step are picked by timing a few
  * choices on the batch (cached per size class) unless fpm(51) sets them.
  * The contour nodes come from fpm(2), fpm(18) and each problem's interval;
@@ -273,8 +274,8 @@ size_t feast_scsr_workspace_min_bytes(int n, int nnz_a, int nnz_b, int m0, const
  * d_ia/d_ja/d_a: 0-based CSR of A in full storage (device); d_ib/d_jb/d_b the
  * same for B or NULL for B = I; d_x: device, column-major n x m0, in/out as x
  * above.  e, res and the scalars are host memory.  d_work: device workspace of
- * at least feast_scsr_workspace_bytes(...) bytes, 256-byte aligned; the
- * library allocates nothing.  Work is enqueued on stream; the call returns
+ * at least feast_scsr_workspace_min_bytes(...) bytes (feast_scsr_workspace_bytes
+ * for the full speed), 256-byte aligned; the library allocates nothing.  Work is enqueued on stream; the call returns
  * once the results are written.  Argument errors as above; the CSR is not
  * re-validated (use feast_scsr_solve for untrusted input). */
 int feast_scsr_solve_dev(int n, int nnz_a, const int* d_ia, const int* d_ja, const double* d_a, int nnz_b,

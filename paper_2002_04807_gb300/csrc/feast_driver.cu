@@ -2183,12 +2183,12 @@ extern "C" int feast_last_profile(double* out)
 
 // ---------------------------------------------------------------- batched driver
 // Many independent problems (FEAST's first level of parallelism: separate
-// search intervals) solved together: one filter launch sequence covers the
-// work items of every unfinished problem, and the Rayleigh-Ritz step is a
-// fixed sequence of batched kernels over all problems.  Both sequences are
-// captured once as CUDA graphs (the COCG step index lives on the device) and
-// replayed every refinement loop; finished problems are switched off by
-// flags in the problem tables.
+// search intervals) solved together: without B a contour pass is one launch per
+// class of sizes (k_krylov.cu), with B the COCG steps cover the work items of
+// every unfinished problem and replay as a captured CUDA graph (the step index
+// lives on the device); the Rayleigh-Ritz step is a fixed sequence of batched
+// kernels over all problems.  Finished problems are switched off by flags in the
+// problem tables.
 namespace {
 
 __global__ void kb_col_to_row(const BProb* pr, const double* xc, double* xr)

@@ -6,18 +6,19 @@
 // problems are flattened into one index space (or work blocks are listed per
 // problem), and a problem table (BProb) gives each problem's sizes and
 // offsets.  A problem whose flag `active` is 0 is skipped, so one launch
-// sequence (and one captured CUDA graph) serves every refinement loop while
-// problems converge at different loops.
+// sequence serves every refinement loop while problems converge at different
+// loops.
 //
 //   b_spmm        Y = A X for every problem's FP64 row-major n x m block
 //   b_gram        partial C = X^T Y per (problem, 64x64 tile pair, row split),
 //                 FP64 tensor cores (mma.sync m8n8k4 f64); b_gram_reduce sums
-//                 the splits in order and symmetrises
+//                 the splits in order and mirrors the upper triangle
 //   b_gemm        C = A V (n x m times m x m) per problem
 //   b_residual    R = A X - B X diag(lambda) and per-column norms
-//   b_reduced     the reduced generalized eigenproblem of one problem per CTA
-//                 (m <= 128): two cyclic Jacobi decompositions in shared and
-//                 global memory, rounds synchronised with __syncthreads
+//   b_reduce_prep the reduced generalized eigenproblem of one problem per CTA
+//                 (m <= 128) up to its standard form S^T A~ S; jacobi_team
+//                 (k_eig.cu) diagonalises it with several CTAs per problem,
+//                 b_reduce_vectors forms V = S W
 #include <algorithm>
 
 #include "chol.cuh"

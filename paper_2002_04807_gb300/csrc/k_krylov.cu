@@ -43,8 +43,9 @@
 // leaves its range for matrices of any size, and a pair of an FP64 pass stops
 // where FP64 recurrences stop it.
 // What bounds it (GB300, 2.07 GHz).  Cached, 7-point 64^3, 150 float columns:
-// 24 ms a pass of 80 steps and 222 (node, step) pairs against 154 ms with COCG
-// per node; a step moves 0.94 GB, A 130 us (3.6 TB/s: the gather's reads
+// 20 ms a pass of 80 steps and 222 (node, step) pairs against 154 ms with COCG
+// per node (a call that has to map the bases' 13.6 GB takes 26 ms among others
+// and 49 alone, with the memory at hand 20.6); a step moves 0.94 GB, A 130 us (3.6 TB/s: the gather's reads
 // through L2, 21 bytes an element, and too few loads in flight), B 88 us (5.4
 // TB/s, DRAM), the two sums 30 us.  Resident, one CTA per 4-column tile
 // (n = 1000): 6.3 us a step, the entries' exchange and two block sums; FP64
@@ -948,7 +949,10 @@ int krylov_rows(int n, int nc) { return krylov_rpc(n, nc); }
 
 int krylov_item_rows(const KrylovPlan& k) { return k.resident ? 32 / k.lanes : kLzBlock; }
 
-// Bytes of Krylov bases beyond which a pass takes its tiles one team at a time.
+// Bytes of Krylov bases that the teams of a pass may hold together: the number of
+// tiles taken at once is limited by it, one team has what it needs whatever that
+// is.  At 64^3 with 150 columns (2.7 GB a tile) all five tiles at once measured 21
+// to 24 ms a pass, one after the other 27; the limit lies just above those five.
 static constexpr double kKrylovMany = 16e9;
 
 // Microseconds of one step of a tile of an n-row problem, by the measured parts of a step on
