@@ -966,9 +966,17 @@ static double krylov_tile_cost(const KrylovPlan& k, bool fp64, int n)
     return 1.8 + passes * (k.resident ? 1.2 : 2.9) * (fp64 ? 4.0 : 1.0) + (k.nc == 1 ? 2.2 : 6.0 + 0.035 * k.nc);
 }
 
+// Steps a problem of n rows may take: its Krylov spaces have at most n
+// dimensions, and a pair that eight times as many steps (and a thousand) have not
+// brought to its tolerance is at its rounding level.  Without this a cap that
+// stands for "none" (fpm(46) = 10^6) planned 17 GB for 100 rows and mapped them in
+// every filter call (36 ms, now 1.6).
+static int krylov_steps(int n, int maxit) { return (int)std::min<long long>(maxit, 8LL * n + 1000); }
+
 // The parts of a plan that follow from its width, for problems of at most n rows.
 static double krylov_size(KrylovPlan& k, bool fp64, int lanes, int n, int ne, int maxit)
 {
+    maxit = krylov_steps(n, maxit);
     k.lanes = lanes;
     k.cols = lanes * (fp64 ? 2 : 4);
     k.nl = std::min(ne, 32);

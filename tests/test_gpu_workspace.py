@@ -92,3 +92,24 @@ def test_batch_on_a_device_without_room_for_the_bases(pkg):
     for r, r0 in zip(got, ref):
         assert r.info == r0.info == 0 and r.M == r0.M > 0
         assert np.abs(r.E[: r.M] - r0.E[: r0.M]).max() <= 1e-9
+
+
+@pytest.mark.parametrize("mixed", [0, 1])
+def test_a_cap_that_stands_for_none_takes_no_memory(pkg, mixed):
+    """fpm(46) = 10^6 on a few hundred rows: the space has no more dimensions than
+    rows, so neither the workspace nor a filter call's own grows with such a cap, and
+    the block is that of a cap the pass does not meet."""
+    A = fw.laplacian_1d(300)
+    csr = [torch.as_tensor(v, device="cuda") for v in (A.indptr, A.indices, A.data)]
+    R = torch.as_tensor(fw.gaussian_block(300, 12, 3), device="cuda")
+    out = []
+    for cap in (400, 1_000_000):
+        f = pkg.feast_init()
+        f[1], f[17], f[41], f[44], f[45] = 8, 100, mixed, (4 if mixed else 10), cap
+        assert pkg.feast_scsr_workspace_bytes(300, A.nnz, 0, 12, f) < 256 << 20
+        Q = torch.zeros_like(R)
+        it = pkg.feast_filter_dev(300, *csr, None, None, None, 12, R, R, torch.zeros(12, dtype=torch.float64, device="cuda"),
+                                  0, f, 0.0, 1.0, Q)
+        assert it < 400
+        out.append(Q.cpu().numpy())
+    assert np.abs(out[0] - out[1]).max() <= 1e-3 * np.abs(out[0]).max()  # both solved to the tolerance
