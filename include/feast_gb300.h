@@ -32,7 +32,8 @@
  *              the M0/2 lowest / largest eigenpairs (feast_scsr_extreme*)
  *      fpm(42) 1: complex FP32 shifted solves (mixed precision), 0: complex FP64
  *      fpm(45) inner solver tolerance 10^-fpm(45) (0..16)
- *      fpm(46) inner solver iteration cap (>= 1)
+ *      fpm(46) inner solver iteration cap (>= 1; one Krylov space per column
+ *              stops at 8 N + 1000 steps where that is less)
  *      fpm(60) output: total number of inner (COCG) iterations
  *    Library options in reserved slots (0 = automatic):
  *      fpm(50) contour nodes solved at once (node batch; with B = I and

@@ -970,7 +970,7 @@ static double krylov_tile_cost(const KrylovPlan& k, bool fp64, int n)
 // dimensions, and a pair that eight times as many steps (and a thousand) have not
 // brought to its tolerance is at its rounding level.  Without this a cap that
 // stands for "none" (fpm(46) = 10^6) planned 17 GB for 100 rows and mapped them in
-// every filter call (36 ms, now 1.6).
+// every filter call (36 ms; now 0.03 GB and 1.5, one COCG per node takes 8.1).
 static int krylov_steps(int n, int maxit) { return (int)std::min<long long>(maxit, 8LL * n + 1000); }
 
 // The parts of a plan that follow from its width, for problems of at most n rows.
