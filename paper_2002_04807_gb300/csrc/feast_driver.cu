@@ -969,7 +969,7 @@ int setup_krylov(const Plan& P, Bufs& B, const Csr& A, cudaStream_t s)
     int* d_wide = (int*)(B.lzmax + 1);
     const bool few = (long long)A.nnz <= 8LL * A.n;
     CK(cudaMemsetAsync(B.lzmax, 0, 2 * sizeof(double), s));
-    CK(launch_krylov_scan(A.n, A.ia, few ? A.ja : nullptr, d_wide, 1, A.v, B.lzmax, s));
+    CK(launch_krylov_scan(A.n, A.nnz, A.ia, few ? A.ja : nullptr, d_wide, 1, A.v, B.lzmax, s));
     if (few) {
         CK(cudaMemcpyAsync(&wide, d_wide, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));

@@ -5,8 +5,6 @@
 #include <stdint.h>
 #include <stddef.h>
 
-#include <cmath>
-
 namespace feast {
 
 // ---------------------------------------------------------------- complex helpers
@@ -189,7 +187,7 @@ struct KrylovArgs {
     void* part;         // [team][2][nc][cols] partial sums (8 bytes)
     double* coef;       // [team][2][maxit + 2][cols] alpha_j, beta_{j+1}
     void* g;            // [team][maxit][cols] combination coefficients (filter precision)
-    void* pair;         // [team][ne][cols] pivot and residual of every pair (LzPair)
+    void* pair;         // [team][ne][cols] shift, pivot and residual of every pair (LzPair)
     int* kstop;         // [team][ne][cols]
     double2* piv;       // [team][cols][maxit][nl]
     unsigned* bar;      // [team][32], zeroed
@@ -214,17 +212,18 @@ int krylov_rows(int n, int nc);  // rows per CTA of the resident form
 int krylov_item_rows(const KrylovPlan& k);
 // Power of two by which the Krylov filter multiplies A and the shifts, so that
 // the steps run on entries near 1 whatever the size of A's (amax: the largest).
-__host__ __device__ inline double krylov_scale(double amax)
+// By its exponent field: every thread that packs an entry takes it.
+__device__ __forceinline__ double krylov_scale(double amax)
 {
-    if (!(amax > 0.0) || !(amax < 1.7e308)) return 1.0;
-    const int e = ilogb(amax);
-    return ldexp(1.0, e < -1000 ? 1000 : -e);
+    const int hi = __double2hiint(amax), field = hi >> 20;  // 2047: infinite or NaN
+    if (field == 2047 || !(amax > 0.0)) return 1.0;
+    return __hiloint2double(min(max(2046 - field, 1), 2023) << 20, 0);
 }
 size_t krylov_layout(const KrylovPlan& k, char* base, KrylovArgs& a);
 // amax (zeroed): the largest |v| of the matrix's entries (parts = 2: of their real
 // and imaginary parts); wide (zeroed), unless ja is null: set when a row needs
-// more than eight packed entries.
-cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, int parts, const double* v, double* amax,
+// more than eight packed entries.  nnz: about how many entries there are.
+cudaError_t launch_krylov_scan(int n, int nnz, const int* ia, const int* ja, int* wide, int parts, const double* v, double* amax,
                                cudaStream_t s);
 cudaError_t launch_krylov_pack(int n, int rpc, const int* ia, const int* ja, const double* av, const double* amax, bool fp64,
                                void* out, cudaStream_t s);

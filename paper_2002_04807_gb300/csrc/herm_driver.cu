@@ -541,7 +541,7 @@ static int h_dev_entry(int n, int nnz_a, const int* d_ia, const int* d_ja, const
         fp.active = 1;
         fp.amax = B.lzmax;
         if (ce == cudaSuccess) ce = cudaMemsetAsync(B.lzmax, 0, sizeof(double), s);
-        if (ce == cudaSuccess) ce = launch_krylov_scan(n, d_ia, nullptr, nullptr, 2, d_a, B.lzmax, s);
+        if (ce == cudaSuccess) ce = launch_krylov_scan(n, nnz_a, d_ia, nullptr, nullptr, 2, d_a, B.lzmax, s);
         if (ce == cudaSuccess) ce = cudaMemcpyAsync(B.lzpp, pp.data(), sizeof(int) * pp.size(), cudaMemcpyHostToDevice, s);
         if (ce == cudaSuccess) ce = cudaMemcpyAsync(B.lzprob, &fp, sizeof(fp), cudaMemcpyHostToDevice, s);
         if (ce == cudaSuccess) ce = launch_krylov_pack_hermitian(n, d_ia, d_ja, A.v, B.lzpp, B.lzmax, P.fp64, B.lzpk, s);

@@ -130,10 +130,12 @@ template <> struct LzSum<double> {
     __device__ __forceinline__ double value() const { return h; }
 };
 
-// A (node, column) pair while it iterates: pivot of z_e - T_j, (|r| / |b|)^2.
+// A (node, column) pair while it iterates: its shift (scaled), pivot of z_e - T_j,
+// (|r| / |b|)^2.
 template <typename T>
-struct alignas(4 * sizeof(T)) LzPair {
-    T re, im, f2, pad;
+struct alignas(sizeof(T) == 4 ? 32 : 16) LzPair {
+    double zr;
+    T zi, re, im, f2;
 };
 
 // ---------------------------------------------------------------- packed rows
@@ -371,7 +373,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                 bt_g[tid] = (double)b;
                 // the pairs of this column: pivot, relative residual, stop step
                 for (int e = 0; e < a.ne; ++e) {
-                    pst[e * COLS + tid] = {T(0), T(0), T(1), T(0)};
+                    pst[e * COLS + tid] = {P.zw[4 * e] * s_zs, (T)(P.zw[4 * e + 1] * s_zs), T(0), T(0), T(1)};
                     kst[e * COLS + tid] = ok ? -1 : 0;
                 }
             }
@@ -631,10 +633,10 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                 int more = 0;
                 for (int pr = tid; pr < npair; pr += kLzThreads) {
                     if (kst[pr] >= 0) continue;
-                    const int e = pr / COLS, cl = pr % COLS;
+                    const int cl = pr % COLS;
                     const LzPair<T> st = pst[pr];
                     const T bn = (T)bt_g[(size_t)j * COLS + cl], bj = (T)bt_g[(size_t)(j - 1) * COLS + cl];
-                    T dr = (T)(P.zw[4 * e] * s_zs - (double)s_al[cl]), di = (T)(P.zw[4 * e + 1] * s_zs);
+                    T dr = (T)(st.zr - (double)s_al[cl]), di = st.zi;
                     if (j > 1) {
                         const T w = bj * bj / (st.re * st.re + st.im * st.im);
                         dr -= w * st.re;
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                     } else if ((double)f2 <= a.tol2) {
                         kst[pr] = j;
                     } else {
-                        pst[pr] = {dr, di, f2, T(0)};
+                        pst[pr] = {st.zr, st.zi, dr, di, f2};
                         more = 1;
                     }
                 }
@@ -838,10 +840,10 @@ __global__ void __launch_bounds__(256) krylov_scan(int n, const int* __restrict_
     if (__syncthreads_or(w) && threadIdx.x == 0) *wide = 1;
 }
 
-cudaError_t launch_krylov_scan(int n, const int* ia, const int* ja, int* wide, int parts, const double* v, double* amax,
+cudaError_t launch_krylov_scan(int n, int nnz, const int* ia, const int* ja, int* wide, int parts, const double* v, double* amax,
                                cudaStream_t s)
 {
-    const int grid = std::max(1, std::min((n + 255) / 256, num_sms() * 8));
+    const int grid = (int)std::max(1LL, std::min<long long>((std::max(n, nnz) + 255LL) / 256, num_sms() * 8));
     krylov_scan<<<grid, 256, 0, s>>>(n, ia, ja, wide, parts, v, (unsigned long long*)amax);
     count_launches(1);
     return cudaGetLastError();
@@ -984,7 +986,7 @@ static double krylov_size(KrylovPlan& k, bool fp64, int lanes, int n, int ne, in
     k.ne = ne;
     k.slot_vecs = (size_t)n * lanes;
     k.team_bytes = ((size_t)maxit + 1) * k.slot_vecs * 16;
-    return (double)k.team_bytes + (double)k.cols * k.nl * 16.0 * maxit + (double)k.cols * (24.0 * maxit + 36.0 * ne);
+    return (double)k.team_bytes + (double)k.cols * k.nl * 16.0 * maxit + (double)k.cols * (24.0 * maxit + 52.0 * ne);
 }
 
 KrylovPlan krylov_plan(bool fp64, bool resident, int n, int m, int ne, int maxit, double max_bytes)
