@@ -131,11 +131,12 @@ template <> struct LzSum<double> {
 };
 
 // A (node, column) pair while it iterates: its shift (scaled), pivot of z_e - T_j,
-// (|r| / |b|)^2.
+// (|r| / |b|)^2; in FP64, where a division is a long chain that every CTA of the
+// team waits for, also 1 / |pivot|^2.
 template <typename T>
 struct alignas(sizeof(T) == 4 ? 32 : 16) LzPair {
     double zr;
-    T zi, re, im, f2;
+    T zi, re, im, f2, rd;
 };
 
 // ---------------------------------------------------------------- packed rows
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                 bt_g[tid] = (double)b;
                 // the pairs of this column: pivot, relative residual, stop step
                 for (int e = 0; e < a.ne; ++e) {
-                    pst[e * COLS + tid] = {P.zw[4 * e] * s_zs, (T)(P.zw[4 * e + 1] * s_zs), T(0), T(0), T(1)};
+                    pst[e * COLS + tid] = {P.zw[4 * e] * s_zs, (T)(P.zw[4 * e + 1] * s_zs), T(0), T(0), T(1), T(0)};
                     kst[e * COLS + tid] = ok ? -1 : 0;
                 }
             }
@@ -638,18 +639,19 @@ __global__ void __launch_bounds__(kLzThreads, RES ? 1 : 2) krylov_filter(KrylovA
                     const T bn = (T)bt_g[(size_t)j * COLS + cl], bj = (T)bt_g[(size_t)(j - 1) * COLS + cl];
                     T dr = (T)(st.zr - (double)s_al[cl]), di = st.zi;
                     if (j > 1) {
-                        const T w = bj * bj / (st.re * st.re + st.im * st.im);
+                        const T w = sizeof(T) == 8 ? bj * bj * st.rd : bj * bj / (st.re * st.re + st.im * st.im);
                         dr -= w * st.re;
                         di += w * st.im;
                     }
                     const T dd = dr * dr + di * di;
-                    const T f2 = st.f2 * (bn * bn / dd);
+                    const T rd = sizeof(T) == 8 ? T(1) / dd : T(0);
+                    const T f2 = st.f2 * (sizeof(T) == 8 ? bn * bn * rd : bn * bn / dd);
                     if (!(dd > T(0)) || !isfinite(f2)) {
                         kst[pr] = j - 1;  // no usable step: keep the last iterate
                     } else if ((double)f2 <= a.tol2) {
                         kst[pr] = j;
                     } else {
-                        pst[pr] = {st.zr, st.zi, dr, di, f2};
+                        pst[pr] = {st.zr, st.zi, dr, di, f2, rd};
                         more = 1;
                     }
                 }
