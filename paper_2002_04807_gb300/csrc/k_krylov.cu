@@ -830,7 +830,13 @@ __global__ void __launch_bounds__(256) krylov_scan(int n, const int* __restrict_
         const unsigned long long x = __shfl_xor_sync(0xffffffffu, most, o);
         if (x > most) most = x;
     }
-    if ((threadIdx.x & 31) == 0 && most > *(volatile unsigned long long*)amax) atomicMax(amax, most);
+    __shared__ unsigned long long s_most[8];
+    if ((threadIdx.x & 31) == 0) s_most[threadIdx.x >> 5] = most;
+    __syncthreads();
+    if (threadIdx.x == 0) {  // atomics on one address queue up: one per CTA
+        for (int i = 1; i < 8; ++i) most = max(most, s_most[i]);
+        if (most > *(volatile unsigned long long*)amax) atomicMax(amax, most);
+    }
     if (!ja) return;
     int w = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -845,7 +851,7 @@ __global__ void __launch_bounds__(256) krylov_scan(int n, const int* __restrict_
 cudaError_t launch_krylov_scan(int n, int nnz, const int* ia, const int* ja, int* wide, int parts, const double* v, double* amax,
                                cudaStream_t s)
 {
-    const int grid = (int)std::max(1LL, std::min<long long>((std::max(n, nnz) + 255LL) / 256, num_sms() * 8));
+    const int grid = (int)std::max(1LL, std::min<long long>((std::max(n, nnz) + 255LL) / 256, num_sms() * 2));
     krylov_scan<<<grid, 256, 0, s>>>(n, ia, ja, wide, parts, v, (unsigned long long*)amax);
     count_launches(1);
     return cudaGetLastError();
